@@ -7,34 +7,19 @@
 namespace gs3 {
 
 constexpr int NT = 128;          // threads per 16x16 tile: two pixels each
-#ifndef BWD_CHUNK_RECORDS
-#define BWD_CHUNK_RECORDS 32
-#endif
-constexpr int BWD_CHUNK = BWD_CHUNK_RECORDS;  // records per backward reduction chunk
-#ifndef BWD_UNROLL
-#define BWD_UNROLL 2
-#endif
 #ifndef FWD_UNROLL
 #define FWD_UNROLL 8
 #endif
-constexpr int kBwdUnroll = BWD_UNROLL, kFwdUnroll = FWD_UNROLL;
-// Optional minimum blocks per SM for the compositing kernels' launch bounds
+constexpr int kFwdUnroll = FWD_UNROLL;
+// Optional minimum blocks per SM for the forward's launch bounds
 // (0: none, the compiler's register choice).
 #ifndef FWD_MIN_BLOCKS
 #define FWD_MIN_BLOCKS 0
-#endif
-#ifndef BWD_MIN_BLOCKS
-#define BWD_MIN_BLOCKS 0
 #endif
 #if FWD_MIN_BLOCKS > 0
 #define FWD_BOUNDS __launch_bounds__(128, FWD_MIN_BLOCKS)
 #else
 #define FWD_BOUNDS __launch_bounds__(128)
-#endif
-#if BWD_MIN_BLOCKS > 0
-#define BWD_BOUNDS __launch_bounds__(128, BWD_MIN_BLOCKS)
-#else
-#define BWD_BOUNDS __launch_bounds__(128)
 #endif
 #ifndef RASTER_WARP_BLOCKS
 #define RASTER_WARP_BLOCKS 1     // 1: each warp owns a compact block of the tile; 0: rows
@@ -122,35 +107,22 @@ __device__ __forceinline__ float2 pair_power2(float2 xy, float4 co, float px, fl
     return __ffma2_rn(make_float2(-0.5f, -0.5f), q, nb);
 }
 
-#ifndef RASTER_LOG2_CONIC
-#define RASTER_LOG2_CONIC 1
-#endif
-// With RASTER_LOG2_CONIC the staged conic is scaled by log2(e) (scale_conic),
-// so pair_power yields the power in base-2 units and G = 2^power comes from
-// one ex2.approx; G, alpha and dL/dpower keep their natural-unit meaning.
-// moments_to_grads takes the unscaled conic (unscale_conic).
+// The staged conic is scaled by log2(e) (scale_conic), so the power comes in
+// base-2 units and G = 2^power from one ex2.approx; alpha and dL/dpower keep
+// their natural-unit meaning.
 constexpr float kLog2e = 1.4426950408889634f, kLn2 = 0.6931471805599453f;
 
 __device__ __forceinline__ float4 scale_conic(float4 co)
 {
-    return RASTER_LOG2_CONIC ? make_float4(co.x * kLog2e, co.y * kLog2e, co.z * kLog2e, co.w) : co;
+    return make_float4(co.x * kLog2e, co.y * kLog2e, co.z * kLog2e, co.w);
 }
 
-__device__ __forceinline__ float4 unscale_conic(float4 co)
-{
-    return RASTER_LOG2_CONIC ? make_float4(co.x * kLn2, co.y * kLn2, co.z * kLn2, co.w) : co;
-}
-
-// G = exp(power) for a power from pair_power on a staged conic.
+// G = 2^power.
 __device__ __forceinline__ float pair_gauss(float power)
 {
-#if RASTER_LOG2_CONIC
     float g;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(g) : "f"(power));
     return g;
-#else
-    return __expf(power);
-#endif
 }
 
 // alpha >= 1/255 (Eq. 4's skip) is tested as power >= pmin on the base-2
@@ -368,62 +340,7 @@ __global__ void FWD_BOUNDS raster_fwd2_kernel(RasterParams p)
     }
 }
 
-// Sum 8 per-lane values over the warp with 9 shuffles: each butterfly stage
-// hands half of the remaining values to the partner lane.  Lane l returns the
-// warp total of value index 4*bit4(l) + 2*bit3(l) + bit2(l) = l >> 2.  With
-// FULL false the last two stages are left out (7 shuffles) and lane l returns
-// the sum of that value over the 8 lanes that share l & 3: the warp total is
-// the sum of lanes 4 (l >> 2) .. 4 (l >> 2) + 3.
-template <bool FULL = true>
-__device__ __forceinline__ float warp_reduce8(const float *v)
-{
-    const int lane = threadIdx.x & 31;
-    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
-    float a[4], b[2];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float send = b4 ? v[i] : v[i + 4];
-        float keep = b4 ? v[i + 4] : v[i];
-        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        float send = b3 ? a[i] : a[i + 2];
-        float keep = b3 ? a[i + 2] : a[i];
-        b[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    float send = b2 ? b[0] : b[1];
-    float c = (b2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, send, 4);
-    if (FULL) {
-        c += __shfl_xor_sync(0xffffffffu, c, 2);
-        c += __shfl_xor_sync(0xffffffffu, c, 1);
-    }
-    return c;
-}
-
-// Record gradients from the tile sums of the moments: with power =
-// -0.5 (A dx^2 + C dy^2) - B dx dy and dx = px - u,
-//   dL/du = A S_x + B S_y,  dL/dv = C S_y + B S_x,
-//   dL/dA = -S_xx / 2,  dL/dB = -S_xy,  dL/dC = -S_yy / 2,
-// S_. = sum of dL/dpower times the offsets' monomials.  h = 0 holds
-// (S_x, S_y, S_xx, S_xy), h = 1 holds (S_yy, r, g, b).
-__device__ __forceinline__ float4 moments_to_grads(float4 s, float4 co, int h)
-{
-    if (h == 0)
-        return make_float4(fmaf(co.x, s.x, co.y * s.y), fmaf(co.z, s.y, co.y * s.x), -0.5f * s.z, -s.w);
-    return make_float4(-0.5f * s.x, s.y, s.z, s.w);
-}
-
-// Reverse with the thread's two vertically adjacent pixels evaluated together
-// in packed FP32 (two lanes of a register pair per instruction).  A pixel
-// that does not take part in a record (past its list end, or the record's
-// power outside [pmin, 0]) gets alpha = 0, which leaves its transmittance,
-// its colour-behind term and the sums exactly as they are.
-struct PixBwd2 {
-    int last0, last1;
-    float2 T, dC0, dC1, dC2, S;
-};
-
+// ------------------------------------------------------------------ reverse
 __device__ __forceinline__ float rcp_approx(float x)
 {
     float r;
@@ -433,222 +350,385 @@ __device__ __forceinline__ float rcp_approx(float x)
 
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
-template <bool WANT_OP, bool STATS>
-__device__ __forceinline__ bool unblend_pair(PixBwd2 &P, int pos, float4 co, float4 c, float2 pw, float pmin,
-                                             float dx, float2 dy, float dxx, float2 dxy, float2 dyy,
-                                             float *v, uint32_t &n_contrib)
+// Reverse: one warp per 8x16 half of a tile, four vertically adjacent pixels a
+// lane as two packed pairs, no barrier anywhere; the warps of a block share
+// nothing.  What bounds it is the instruction issue of the pair arithmetic
+// and, at small images, the longest tile.  Why it is cut this way (250K
+// Gaussians, four 1352x1014 views / 50K, eight 480x360 views, one launch, by
+// CUPTI):
+//  - the sums over pixels are taken with the lanes turned.  While a chunk of
+//    BWD_CHUNK records is walked, lane = pixel column, and each lane leaves
+//    the sums over its own four pixels (of dL/dpower times 1, dy, dy^2 and of
+//    the colour gradient) in shared memory; then lane = (record, pixels), and
+//    four lanes add up a record's 32 columns.  A shuffle butterfly per record
+//    for each pixel pair, summed over a tile's warps behind two barriers a
+//    chunk, took half of the kernel's instructions: 922 / 294 us, against
+//    664 / 203 us now.
+//  - each warp keeps, of the tile's list, the records that can reach its own
+//    half (staged_hits), which the former per-tile staging could not use.
+//  - four pixels a lane share a record's loads and column offset: two pixels
+//    a lane (8x8 per warp) ran into the shared-memory pipe (79 % of its
+//    wavefronts) at 731 / 188 us.
+//  - no branch on "no lane takes part": the records of a chunk run as one
+//    straight line, so that their independent parts overlap (715 -> 667 us).
+//  - tiles whose list is long go first (kHeavyList).
+constexpr int BWD_WARPS = 4;                 // warps of a block (two tiles); 1, 2 and 4 measured within 2 %
+constexpr int BWD_CHUNK = 8;                 // records of a turned sum
+constexpr int BWD_ROW = 36;                  // lanes' places of a record: two records of a quarter warp meet different banks
+constexpr int BWD_QUEUE = 32 + BWD_CHUNK;    // staged records of a warp: a batch and what was left of the one before
+constexpr int BWD_TEST = 128;                // records of a bin's list tested at a time (tiles without a list)
+// A block that walks one long list alone at the end of the launch keeps the
+// other SMs waiting, so the grid has two layers: the first takes the tiles
+// with at least this many records (and those without a list), the second the
+// others; a block of the other kind returns at once.  Lists of the headline
+// workload: median 70, 90 % below 219, longest over 1 000.  50K Gaussians in
+// 480x360 views 241 -> 205 us, the headline batch 666 -> 662 us (192: 218 /
+// 665, 384: 212 / 685).
+constexpr int kHeavyList = 256;
+
+struct PixBwd4 {
+    int last[4];
+    float2 T[2], dC0[2], dC1[2], dC2[2], nS[2];   // nS: minus dL/dC . (colour behind)
+};
+
+struct BwdWarp {
+    float4 sum4[BWD_CHUNK][BWD_ROW];   // per record and lane, over its pixels: S, S_y, S_yy, red
+    float2 sum2[BWD_CHUNK][BWD_ROW];   // green, blue
+    float4 xyt[BWD_QUEUE];             // mean, threshold power, list position
+    float4 co[BWD_QUEUE];              // conic in base-2 units, and minus the opacity
+    float4 rgbg[BWD_QUEUE];            // colour, Gaussian
+    uint2 cand[BWD_TEST + 32];         // tiles without a list: records whose rectangle holds the tile
+};
+
+// Can a staged record reach alpha >= 1/255 at some centre of the 8x16 pixels
+// from (cx, cy) on?  As ellipse_hits_tile, in the staged units (the negated
+// power, base 2), with the evaluation's rounding taken off the form:
+// a record dropped here is one that every pixel of the warp skips.
+__device__ __forceinline__ bool staged_hits(float4 xyt, float4 co, float cx, float cy)
 {
-    const bool in0 = pos < P.last0 && pw.x <= 0.f && pw.x >= pmin;
-    const bool in1 = pos < P.last1 && pw.y <= 0.f && pw.y >= pmin;
-    if (!(in0 || in1)) return false;
-    if (STATS) n_contrib += (uint32_t)in0 + (uint32_t)in1;
-    const float g0 = in0 ? pair_gauss(pw.x) : 0.f, g1 = in1 ? pair_gauss(pw.y) : 0.f;
-    const float2 araw = __fmul2_rn(f2(co.w), make_float2(g0, g1));
-    const float2 alpha = make_float2(fminf(kAlphaCap, araw.x), fminf(kAlphaCap, araw.y));
-    const float2 om = __ffma2_rn(alpha, f2(-1.f), f2(1.f));   // 1 - alpha
-    P.T = __fmul2_rn(P.T, make_float2(in0 ? rcp_approx(om.x) : 1.f, in1 ? rcp_approx(om.y) : 1.f));
-    const float2 w = __fmul2_rn(alpha, P.T);
-    const float2 c0 = __fmul2_rn(P.dC0, w), c1 = __fmul2_rn(P.dC1, w), c2 = __fmul2_rn(P.dC2, w);
-    v[5] = c0.x + c0.y;
-    v[6] = c1.x + c1.y;
-    v[7] = c2.x + c2.y;
-    float2 t = __fmul2_rn(P.dC0, f2(c.x));
-    t = __ffma2_rn(P.dC1, f2(c.y), t);
-    t = __ffma2_rn(P.dC2, f2(c.z), t);
-    const float2 diff = __ffma2_rn(P.S, f2(-1.f), t);          // dC . c - S
-    const float2 dalpha = __fmul2_rn(P.T, diff);
-    P.S = __ffma2_rn(alpha, diff, P.S);
-    // moments of dL/dpower over the pair offsets (no gradient through a capped alpha)
-    float2 dpow = __fmul2_rn(dalpha, alpha);
-    if (!(araw.x < kAlphaCap)) dpow.x = 0.f;
-    if (!(araw.y < kAlphaCap)) dpow.y = 0.f;
-    const float sd = dpow.x + dpow.y;
-    v[0] = sd * dx;
-    v[2] = sd * dxx;
-    const float2 m1 = __fmul2_rn(dpow, dy), m3 = __fmul2_rn(dpow, dxy), m4 = __fmul2_rn(dpow, dyy);
-    v[1] = m1.x + m1.y;
-    v[3] = m3.x + m3.y;
-    v[4] = m4.x + m4.y;
-    if (WANT_OP) {
-        const float2 gm = make_float2(araw.x < kAlphaCap ? g0 : 0.f, araw.y < kAlphaCap ? g1 : 0.f);
-        const float2 op = __fmul2_rn(dalpha, gm);
-        v[8] = op.x + op.y;
+    const float tau = xyt.z + 0.0075f;
+    const float xa = cx - xyt.x, xb = xa + 7.f, ya = cy - xyt.y, yb = ya + 15.f;
+    if (xa <= 0.f && xb >= 0.f && ya <= 0.f && yb >= 0.f) return true;
+    const float A = 0.5f * co.x, B = co.y, C = 0.5f * co.z;   // A dx^2 + B dx dy + C dy^2
+    const float bA = 0.5f * B * __frcp_rn(A), bC = 0.5f * B * __frcp_rn(C);
+    auto form = [&](float dx, float dy) {
+        const float s = A * dx * dx + C * dy * dy;
+        return fmaf(-1e-6f, s, fmaf(B * dx, dy, s));
+    };
+    auto qx = [&](float dx) { return form(dx, fminf(fmaxf(-bC * dx, ya), yb)); };
+    auto qy = [&](float dy) { return form(fminf(fmaxf(-bA * dy, xa), xb), dy); };
+    return fminf(fminf(qx(xa), qx(xb)), fminf(qy(ya), qy(yb))) <= tau;
+}
+
+// Weight times dL/dC.  GUARD: a pixel that takes no part (weight 0) gives 0
+// even where its dL/dC is not finite.
+template <bool GUARD>
+__device__ __forceinline__ float2 weigh(float2 w, float2 d)
+{
+    return GUARD ? make_float2(w.x == 0.f ? 0.f : w.x * d.x, w.y == 0.f ? 0.f : w.y * d.y) : __fmul2_rn(w, d);
+}
+template <bool GUARD>
+__device__ __forceinline__ float2 weigh(float2 w, float2 d, float2 a)
+{
+    return GUARD ? __fadd2_rn(a, weigh<true>(w, d)) : __ffma2_rn(w, d, a);
+}
+
+// The chunk's cnt records from slot `head` on at the warp's pixels, back to
+// front (slots past cnt hold records that take part nowhere), and their
+// gradients added to p.grads.
+//
+// power is carried negated, np = (A dx^2 + C dy^2) / 2 + B dx dy, with the
+// forward's roundings (negation is exact; the sum is written as a fused
+// multiply-add by 0.5 because the compiler contracts a packed product and a
+// packed sum, which would round, and decide, differently).  A pixel takes part
+// when np is in [0, threshold]: one unsigned comparison of the bit patterns,
+// which a negative or NaN np fails.  A pixel that takes no part gets
+// alpha = 0 and no difference, which leaves its transmittance, its
+// colour-behind term and the sums exactly as they are.
+//
+// Record gradients from the moments: with power = -(A dx^2 + C dy^2) / 2 -
+// B dx dy and dx = px - u,
+//   dL/du = A S_x + B S_y,  dL/dv = C S_y + B S_x,
+//   dL/dA = -S_xx / 2,  dL/dB = -S_xy,  dL/dC = -S_yy / 2,
+// S_. = sum of dL/dpower times the offsets' monomials; the sums below are of
+// -dL/dpower and of minus the weight.
+template <bool WANT_OP, bool STATS, bool GUARD>
+__device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, PixBwd4 &P, int head, int cnt, float pxf,
+                                          const float2 (&pyf)[2], float cx0, int64_t vb, uint32_t &n_tested,
+                                          uint32_t &n_contrib)
+{
+    constexpr unsigned all = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+#pragma unroll 4
+    for (int i = 0; i < BWD_CHUNK; ++i) {
+        const float4 xyt = S.xyt[head + i];
+        const float4 co = S.co[head + i];
+        const float4 c = S.rgbg[head + i];
+        const int pos = __float_as_int(xyt.w);
+        const uint32_t thr = __float_as_uint(xyt.z);
+        const float dx = __fsub_rn(pxf, xyt.x);
+        const float axx = __fmul_rn(co.x, __fmul_rn(dx, dx));
+        float2 dy[2], dyy[2], nd[2], nw[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            dy[h] = __fadd2_rn(pyf[h], f2(-xyt.y));
+            dyy[h] = __fmul2_rn(dy[h], dy[h]);
+            const float2 q = __ffma2_rn(f2(co.z), dyy[h], f2(axx));
+            const float2 np = __ffma2_rn(f2(0.5f), q, __fmul2_rn(f2(co.y), __fmul2_rn(f2(dx), dy[h])));
+            const bool in0 = pos < P.last[2 * h] && __float_as_uint(np.x) <= thr;
+            const bool in1 = pos < P.last[2 * h + 1] && __float_as_uint(np.y) <= thr;
+            if (STATS) {
+                n_tested += (pos < P.last[2 * h]) + (pos < P.last[2 * h + 1]);
+                n_contrib += (uint32_t)in0 + (uint32_t)in1;
+            }
+            // minus alpha, before and after the cap
+            float2 raw = __fmul2_rn(f2(co.w), make_float2(pair_gauss(-np.x), pair_gauss(-np.y)));
+            raw.x = in0 ? raw.x : 0.f;
+            raw.y = in1 ? raw.y : 0.f;
+            const float2 na = make_float2(fmaxf(-kAlphaCap, raw.x), fmaxf(-kAlphaCap, raw.y));
+            const float2 om = __fadd2_rn(na, f2(1.f));
+            P.T[h] = __fmul2_rn(P.T[h], make_float2(rcp_approx(om.x), rcp_approx(om.y)));
+            nw[h] = __fmul2_rn(na, P.T[h]);
+            float2 t = __fmul2_rn(P.dC0[h], f2(c.x));
+            t = __ffma2_rn(P.dC1[h], f2(c.y), t);
+            t = __ffma2_rn(P.dC2[h], f2(c.z), t);
+            float2 diff = __fadd2_rn(t, P.nS[h]);   // dC . c - S
+            diff.x = in0 ? diff.x : 0.f;
+            diff.y = in1 ? diff.y : 0.f;
+            P.nS[h] = __ffma2_rn(na, diff, P.nS[h]);
+            nd[h] = __fmul2_rn(__fmul2_rn(P.T[h], diff), na);
+            if (co.w <= -kAlphaCap) {   // no gradient through a capped alpha
+                if (!(raw.x > -kAlphaCap)) nd[h].x = 0.f;
+                if (!(raw.y > -kAlphaCap)) nd[h].y = 0.f;
+            }
+        }
+        const float2 s = __fadd2_rn(nd[0], nd[1]);
+        const float2 sy = __ffma2_rn(nd[1], dy[1], __fmul2_rn(nd[0], dy[0]));
+        const float2 syy = __ffma2_rn(nd[1], dyy[1], __fmul2_rn(nd[0], dyy[0]));
+        const float2 r = weigh<GUARD>(nw[1], P.dC0[1], weigh<GUARD>(nw[0], P.dC0[0]));
+        const float2 g = weigh<GUARD>(nw[1], P.dC1[1], weigh<GUARD>(nw[0], P.dC1[0]));
+        const float2 b = weigh<GUARD>(nw[1], P.dC2[1], weigh<GUARD>(nw[0], P.dC2[0]));
+        S.sum4[i][lane] = make_float4(s.x + s.y, sy.x + sy.y, syy.x + syy.y, r.x + r.y);
+        S.sum2[i][lane] = make_float2(g.x + g.y, b.x + b.y);
     }
-    return true;
+    __syncwarp();
+    // lane = (record tr, columns th and th + 4)
+    const int tr = lane >> 2, th = lane & 3, j = head + tr;
+    const float4 xyt = S.xyt[j];
+    const float4 co = S.co[j];
+    float s0 = 0.f, sx = 0.f, sy = 0.f, sxx = 0.f, sxy = 0.f, syy = 0.f, r = 0.f;
+    float2 gb = f2(0.f);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        float2 a = f2(0.f), y = f2(0.f);   // the column's (S, S_y) and (S_yy, red)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 e = S.sum4[tr][8 * q + 4 * i + th];
+            a = __fadd2_rn(a, make_float2(e.x, e.y));
+            y = __fadd2_rn(y, make_float2(e.z, e.w));
+            gb = __fadd2_rn(gb, S.sum2[tr][8 * q + 4 * i + th]);
+        }
+        const float dx = __fsub_rn(cx0 + (float)(4 * i + th), xyt.x);
+        const float adx = a.x * dx;
+        s0 += a.x;
+        sx += adx;
+        sxx = fmaf(adx, dx, sxx);
+        sy += a.y;
+        sxy = fmaf(a.y, dx, sxy);
+        syy += y.x;
+        r += y.y;
+    }
+    // the record's four lanes exchange halves: lane th ends with two of the 8 sums
+    float v[8] = {sx, sy, sxx, sxy, syy, r, gb.x, gb.y};
+    const bool up = th & 2, up1 = th & 1;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float send = up ? v[q] : v[q + 4];
+        v[q] = (up ? v[q + 4] : v[q]) + __shfl_xor_sync(all, send, 2);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const float send = up1 ? v[q] : v[q + 2];
+        v[q] = (up1 ? v[q + 2] : v[q]) + __shfl_xor_sync(all, send, 1);
+    }
+    const float A = co.x * -kLn2, B = co.y * -kLn2, C = co.z * -kLn2;
+    const int64_t gi = vb + __float_as_uint(S.rgbg[j].w);
+    float2 gq = make_float2(th == 3 ? -v[0] : 0.5f * v[0], th == 1 ? v[1] : -v[1]);
+    if (th == 0) gq = make_float2(fmaf(A, v[0], B * v[1]), fmaf(C, v[1], B * v[0]));
+    if (tr < cnt && (v[0] != 0.f || v[1] != 0.f))
+        atomicAdd(reinterpret_cast<float2 *>(p.grads + 8 * gi + 2 * th), gq);
+    if (WANT_OP) {
+        // sum of dL/dalpha G = (sum of dL/dpower) / o, as dL/dpower = dL/dalpha o G
+        s0 += __shfl_xor_sync(all, s0, 1);
+        s0 += __shfl_xor_sync(all, s0, 2);
+        if (tr < cnt && th == 0 && s0 != 0.f) atomicAdd(p.d_opacity + gi, s0 / co.w);
+    }
+    __syncwarp();
 }
 
 template <bool WANT_OP, bool BINNED, bool STATS>
-__global__ void BWD_BOUNDS raster_bwd2_kernel(RasterParams p)
+__global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams p)
 {
-    constexpr int NW = NT / 32;
-    constexpr int NV = WANT_OP ? 9 : 8;
-    __shared__ float4 s_xy[NT];
-    __shared__ float4 s_co[NT];
-    __shared__ float4 s_rgbk[NT];  // colour and (bit pattern of) the list position
-    __shared__ uint32_t s_g[NT];
-    __shared__ int s_wcnt[NW];
-    __shared__ float4 s_part[NW][BWD_CHUNK][8];
-    __shared__ float s_pop[WANT_OP ? NW : 1][BWD_CHUNK];
-    __shared__ int s_max;
-    const int tile = blockIdx.x, view = blockIdx.y;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ BwdWarp s_warp[BWD_WARPS];
+    constexpr unsigned all = 0xffffffffu;
+    BwdWarp &S = s_warp[threadIdx.x >> 5];
+    const int view = blockIdx.y, lane = threadIdx.x & 31;
+    const int unit = blockIdx.x * BWD_WARPS + (threadIdx.x >> 5);
+    const int tile = unit >> 1;
+    if (tile >= p.tx * p.ty) return;
+    const int64_t tg = (int64_t)view * (p.tx * p.ty) + tile;
+    // with the forward's list of the tile, its records are staged straight
+    // from it (list order is position order); otherwise the bin's list is
+    // tested again
+    const int listed = p.tl_rec ? p.tl_cnt[tg] : -1;
+    const bool heavy = listed < 0 || listed >= kHeavyList;
+    if (listed == 0 || heavy != (blockIdx.z == 0)) return;
     const int tx_t = tile % p.tx, ty_t = tile / p.tx;
-    int px, py0;
-    tile_pixel(tid, 2, 0, px, py0);
-    px += tx_t * 16;
-    py0 += ty_t * 16;
+    const int wx = tx_t * 16 + (unit & 1) * 8, wy = ty_t * 16;
+    const int px = wx + (lane & 7), py0 = wy + (lane >> 3) * 4;
+    const float cx0 = (float)wx + 0.5f, cy0 = (float)wy + 0.5f;   // centre of the warp's first pixel
     const float pxf = (float)px + 0.5f;
-    const float2 pyf = make_float2((float)py0 + 0.5f, (float)py0 + 1.5f);
-    const int binid = (ty_t / p.bin) * p.bins_x + tx_t / p.bin;
-    const uint2 range = p.ranges[(int64_t)view * p.bins + binid];
+    const float2 pyf[2] = {make_float2((float)py0 + 0.5f, (float)py0 + 1.5f),
+                           make_float2((float)py0 + 2.5f, (float)py0 + 3.5f)};
     const int64_t vb = (int64_t)view * p.n;
     const int64_t HW = (int64_t)p.H * p.W;
-    PixBwd2 P;
-    P.last0 = P.last1 = 0;
-    float Tq[2] = {1.f, 1.f}, d0[2] = {0.f, 0.f}, d1[2] = {0.f, 0.f}, d2[2] = {0.f, 0.f}, Sq[2] = {0.f, 0.f};
-    int lq[2] = {0, 0};
+    PixBwd4 P;
+    bool bad = false;
+    {
+        float T[4], d0[4], d1[4], d2[4], ns[4];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const int py = py0 + k;
-        if (px < p.W && py < p.H) {
-            int64_t pix = (int64_t)view * HW + (int64_t)py * p.W + px;
-            lq[k] = p.last[pix];
-            Tq[k] = p.T_final[pix];
-            const float *di = p.d_img + (int64_t)view * 3 * HW + (int64_t)py * p.W + px;
-            d0[k] = di[0];
-            d1[k] = di[HW];
-            d2[k] = di[2 * HW];
-            Sq[k] = fmaf(d2[k], p.bg2, fmaf(d1[k], p.bg1, d0[k] * p.bg0));
+        for (int k = 0; k < 4; ++k) {
+            const int py = py0 + k;
+            P.last[k] = 0;
+            T[k] = 1.f;
+            d0[k] = d1[k] = d2[k] = 0.f;
+            if (px < p.W && py < p.H) {
+                const int64_t pix = (int64_t)view * HW + (int64_t)py * p.W + px;
+                const float *di = p.d_img + (int64_t)view * 3 * HW + (int64_t)py * p.W + px;
+                P.last[k] = p.last[pix];
+                T[k] = p.T_final[pix];
+                d0[k] = di[0];
+                d1[k] = di[HW];
+                d2[k] = di[2 * HW];
+            }
+            ns[k] = -fmaf(d2[k], p.bg2, fmaf(d1[k], p.bg1, d0[k] * p.bg0));
+            bad |= !isfinite(d0[k] + d1[k] + d2[k]);
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            P.T[h] = make_float2(T[2 * h], T[2 * h + 1]);
+            P.dC0[h] = make_float2(d0[2 * h], d0[2 * h + 1]);
+            P.dC1[h] = make_float2(d1[2 * h], d1[2 * h + 1]);
+            P.dC2[h] = make_float2(d2[2 * h], d2[2 * h + 1]);
+            P.nS[h] = make_float2(ns[2 * h], ns[2 * h + 1]);
         }
     }
-    P.last0 = lq[0];
-    P.last1 = lq[1];
-    P.T = make_float2(Tq[0], Tq[1]);
-    P.dC0 = make_float2(d0[0], d0[1]);
-    P.dC1 = make_float2(d1[0], d1[1]);
-    P.dC2 = make_float2(d2[0], d2[1]);
-    P.S = make_float2(Sq[0], Sq[1]);
-    const int mylast = max(lq[0], lq[1]);
-    if (tid == 0) s_max = 0;
-    __syncthreads();
-    if (mylast > 0) atomicMax(&s_max, mylast);
-    __syncthreads();
-    const int maxlast = s_max;
+    const bool guard = __any_sync(all, bad);
+    const int wlast = __reduce_max_sync(all, max(max(P.last[0], P.last[1]), max(P.last[2], P.last[3])));
+    if (wlast == 0) return;
     uint32_t n_tested = 0, n_contrib = 0;
-    // with the forward's list of the tile, its records are staged straight
-    // from it (list order is position order; the few past maxlast are
-    // skipped by the position test); otherwise the bin's list is tested again
-    const int64_t tg = (int64_t)view * gridDim.x + tile;
-    const int listed = p.tl_rec ? p.tl_cnt[tg] : -1;
-    for (int hi = listed >= 0 ? listed : maxlast; hi > 0; hi -= NT) {
-        const int lo = max(0, hi - NT);
-        int64_t o = 0;
-        uint32_t g = 0;
-        int k = 0;
-        bool keep = false;
-        float2 m;
-        float4 co;
-        int cnt, slot;
-        if (listed >= 0) {
-            if (lo + tid < hi) {
-                const uint2 e = p.tl_rec[tg * p.tl_cap + lo + tid];
-                g = e.x;
-                k = (int)e.y;
-                o = vb + g;
-                m = p.mean2d[o];
-                co = p.conic_op[o];
-                keep = true;
-            }
-            cnt = hi - lo;
-            slot = keep ? tid : -1;
-        } else {
-            k = lo + tid;
-            if (k < hi) {
-                g = p.vals[range.x + k];
-                o = vb + g;
-                keep = keep_record<BINNED>(p, o, tx_t, ty_t, m, co);
-            }
-            slot = compact_slot<NT>(keep, s_wcnt, cnt);
-        }
-        if (slot >= 0) {
-            s_g[slot] = g;
-            s_xy[slot] = make_float4(m.x, m.y, -__log2f(255.f * co.w), 0.f);
-            s_co[slot] = scale_conic(co);
-            s_rgbk[slot] = make_float4(p.rgb[3 * o], p.rgb[3 * o + 1], p.rgb[3 * o + 2],
-                                       __int_as_float(k));
-        }
-        __syncthreads();
-        for (int chi = cnt; chi > 0; chi -= BWD_CHUNK) {
-            const int clo = max(0, chi - BWD_CHUNK);
-#pragma unroll kBwdUnroll
-            for (int j = chi - 1; j >= clo; --j) {
-                float v[NV];
-                const float4 c = s_rgbk[j];
-                const int pos = __float_as_int(c.w);
-                bool contrib = false;
-                if (pos < mylast) {
-                    const float4 xyp = s_xy[j];
-                    const float4 cc = s_co[j];
-                    float dx, dxx;
-                    float2 dy, dxy, dyy;
-                    const float2 pw = pair_power2(make_float2(xyp.x, xyp.y), cc, pxf, pyf, dx, dy, dxx, dxy, dyy);
-                    if (STATS) n_tested += (pos < P.last0) + (pos < P.last1);
-                    contrib = unblend_pair<WANT_OP, STATS>(P, pos, cc, c, pw, xyp.z, dx, dy, dxx, dxy,
-                                                           dyy, v, n_contrib);
-                }
-                if (!contrib) {
+    const uint2 *rec = p.tl_rec + tg * p.tl_cap;
+    uint32_t first = 0;
+    if (listed < 0) {
+        const int binid = (ty_t / p.bin) * p.bins_x + tx_t / p.bin;
+        first = p.ranges[(int64_t)view * p.bins + binid].x;
+    }
+    int head = 0, have = 0;     // the queue: its first record's slot (a multiple of BWD_CHUNK) and its length
+    int cand0 = 0, cands = 0;   // tiles without a list: the candidates not yet staged
+    int left = listed >= 0 ? listed : wlast;
+    while (left > 0 || cands > 0 || have > 0) {
+        // stage batches of 32 records, back to front, until a chunk is full
+        while ((left > 0 || cands > 0) && have < BWD_CHUNK) {
+            uint2 e = make_uint2(0u, 0x7fffffffu);   // (Gaussian, position)
+            if (listed >= 0) {
+                const int i = left - 1 - lane;
+                if (i >= 0) e = rec[i];
+                left -= 32;
+            } else {
+                // a bin's list can hold tens of thousands of records, few of
+                // them this tile's: their rectangles are tested BWD_TEST at a
+                // time, every load of a test in flight at once (one test of
+                // 32 after the other made a single such tile the launch's
+                // longest: 832 -> 667 us)
+                if (cands < 32 && left > 0) {
+                    if (lane < cands) e = S.cand[cand0 + lane];
+                    __syncwarp();
+                    if (lane < cands) S.cand[lane] = e;
+                    cand0 = 0;
+                    while (cands < 32 && left > 0) {
+                        constexpr int U = BWD_TEST / 32;
+                        uint32_t g[U];
+                        int r[U];
+                        float2 m[U];
 #pragma unroll
-                    for (int q = 0; q < NV; ++q) v[q] = 0.f;
-                }
-                float *part = reinterpret_cast<float *>(&s_part[warp][j - clo][0]);
-                if (__any_sync(0xffffffffu, contrib)) {
-                    part[lane] = warp_reduce8<false>(v);
-                    if (WANT_OP) {
-                        float ro = warp_sum(v[NV - 1]);
-                        if (lane == 0) s_pop[warp][j - clo] = ro;
+                        for (int u = 0; u < U; ++u) {
+                            const int i = left - 1 - lane - 32 * u;
+                            g[u] = i >= 0 ? p.vals[first + i] : 0u;
+                        }
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            const bool ok = left - 1 - lane - 32 * u >= 0;
+                            r[u] = ok ? (BINNED ? p.radius[vb + g[u]] : 1) : 0;
+                            m[u] = ok ? p.mean2d[vb + g[u]] : make_float2(0.f, 0.f);
+                        }
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            bool in = r[u] > 0;
+                            if (BINNED && in) {
+                                int x0, y0, x1, y1;
+                                tile_rect(m[u].x, m[u].y, r[u], p.tx, p.ty, x0, y0, x1, y1);
+                                in = tx_t >= x0 && tx_t < x1 && ty_t >= y0 && ty_t < y1;
+                            }
+                            const unsigned b = __ballot_sync(all, in);
+                            if (in)
+                                S.cand[cands + __popc(b & ((1u << lane) - 1u))] =
+                                    make_uint2(g[u], (uint32_t)(left - 1 - lane - 32 * u));
+                            cands += __popc(b);
+                        }
+                        left -= BWD_TEST;
                     }
-                } else {
-                    part[lane] = 0.f;
-                    if (WANT_OP && lane == 0) s_pop[warp][j - clo] = 0.f;
+                    __syncwarp();
                 }
+                const int take = min(cands, 32);
+                e = lane < take ? S.cand[cand0 + lane] : make_uint2(0u, 0x7fffffffu);
+                cand0 += take;
+                cands -= take;
             }
-            __syncthreads();
-            const int ccnt = chi - clo;
-            if (tid < 4 * ccnt) {
-                // four threads a record, two moments each
-                const int j = tid >> 2, q = (tid & 3) * 2;
-                float2 sum = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int w = 0; w < NW; ++w) {
-                    const float4 a = s_part[w][j][q], b = s_part[w][j][q + 1];
-                    sum.x += (a.x + a.y) + (a.z + a.w);
-                    sum.y += (b.x + b.y) + (b.z + b.w);
-                }
-                if (sum.x != 0.f || sum.y != 0.f) {
-                    float2 gq;
-                    if (q == 0) {
-                        const float4 co = unscale_conic(s_co[clo + j]);
-                        gq = make_float2(fmaf(co.x, sum.x, co.y * sum.y), fmaf(co.z, sum.y, co.y * sum.x));
-                    } else if (q == 2) {
-                        gq = make_float2(-0.5f * sum.x, -sum.y);
-                    } else if (q == 4) {
-                        gq = make_float2(-0.5f * sum.x, sum.y);
-                    } else {
-                        gq = sum;
-                    }
-                    atomicAdd(reinterpret_cast<float2 *>(p.grads + 8 * (vb + s_g[clo + j]) + q), gq);
-                }
+            bool keep = (int)e.y < wlast;
+            float4 xyt, co;
+            if (keep) {
+                const float2 m = p.mean2d[vb + e.x];
+                co = p.conic_op[vb + e.x];
+                xyt = make_float4(m.x, m.y, __log2f(255.f * co.w), __uint_as_float(e.y));
+                co = scale_conic(co);
+                co.w = -co.w;
+                keep = xyt.z >= 0.f && staged_hits(xyt, co, cx0, cy0);
             }
-            if (WANT_OP) {
-                for (int j = tid; j < ccnt; j += NT) {
-                    float sum = 0.f;
-#pragma unroll
-                    for (int w = 0; w < NW; ++w) sum += s_pop[w][j];
-                    if (sum != 0.f) atomicAdd(p.d_opacity + vb + s_g[clo + j], sum);
-                }
+            const unsigned kept = __ballot_sync(all, keep);
+            if (keep) {
+                int q = head + have + __popc(kept & ((1u << lane) - 1u));
+                if (q >= BWD_QUEUE) q -= BWD_QUEUE;
+                const float *c = p.rgb + 3 * (vb + e.x);
+                S.xyt[q] = xyt;
+                S.co[q] = co;
+                S.rgbg[q] = make_float4(c[0], c[1], c[2], __uint_as_float(e.x));
             }
-            __syncthreads();
+            have += __popc(kept);
         }
+        if (have == 0) break;
+        const int cnt = min(have, BWD_CHUNK);
+        if (lane >= cnt && lane < BWD_CHUNK) {   // the last chunk's missing records take part nowhere
+            S.xyt[head + lane] = make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fffffff));
+            S.co[head + lane] = S.rgbg[head + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        __syncwarp();
+        if (guard)
+            bwd_chunk<WANT_OP, STATS, true>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_tested, n_contrib);
+        else
+            bwd_chunk<WANT_OP, STATS, false>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_tested, n_contrib);
+        head += BWD_CHUNK;
+        if (head == BWD_QUEUE) head = 0;
+        have -= cnt;
     }
     if (STATS) flush_stats(p.stats, n_tested, n_contrib);
 }
@@ -694,12 +774,15 @@ static gs_status fill(const gs_projected *proj, int64_t n, int V, int W, int H, 
 }
 
 template <bool WANT_OP, bool BINNED>
-static void launch_bwd(const RasterParams &p, dim3 grid, cudaStream_t s)
+static void launch_bwd(const RasterParams &p, cudaStream_t s)
 {
+    // two warps a tile; the second layer takes the tiles with short lists
+    // (without lists every tile is the first layer's)
+    const dim3 grid((unsigned)ceil_div(2 * p.tx * p.ty, BWD_WARPS), p.V, p.tl_rec ? 2 : 1);
     if (p.stats)
-        raster_bwd2_kernel<WANT_OP, BINNED, true><<<grid, NT, 0, s>>>(p);
+        raster_bwd_kernel<WANT_OP, BINNED, true><<<grid, 32 * BWD_WARPS, 0, s>>>(p);
     else
-        raster_bwd2_kernel<WANT_OP, BINNED, false><<<grid, NT, 0, s>>>(p);
+        raster_bwd_kernel<WANT_OP, BINNED, false><<<grid, 32 * BWD_WARPS, 0, s>>>(p);
 }
 
 }  // namespace gs3
@@ -757,15 +840,14 @@ extern "C" gs_status gs_raster_bwd(const gs_projected *proj, int64_t n, int V, i
     p.grads = grads;
     p.d_opacity = d_opacity;
     p.stats = reinterpret_cast<unsigned long long *>(d_stats);
-    dim3 grid(p.tx * p.ty, V);
     note_launch();
     if (d_opacity && bin > 1)
-        launch_bwd<true, true>(p, grid, s);
+        launch_bwd<true, true>(p, s);
     else if (d_opacity)
-        launch_bwd<true, false>(p, grid, s);
+        launch_bwd<true, false>(p, s);
     else if (bin > 1)
-        launch_bwd<false, true>(p, grid, s);
+        launch_bwd<false, true>(p, s);
     else
-        launch_bwd<false, false>(p, grid, s);
+        launch_bwd<false, false>(p, s);
     return launch_status("gs_raster_bwd");
 }
