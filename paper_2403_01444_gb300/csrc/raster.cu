@@ -1,50 +1,13 @@
-// Front-to-back alpha compositing (Section 3.2, Eq. 4) and its reverse.
-// One 16x16 tile per 128-thread block, two vertically adjacent pixels per
-// thread evaluated together in packed FP32; the tile's depth-sorted records
-// are staged through shared memory in batches of 128.
+// Front-to-back alpha compositing (Section 3.2, Eq. 4) and its reverse.  Both
+// evaluate vertically adjacent pixels in pairs, in packed FP32, on a tile's
+// depth-sorted records staged through shared memory.  The arithmetic of a
+// pixel is written with explicit roundings so that both passes, and every
+// way of cutting the work, take bit-identical decisions.
 #include "common.cuh"
 
 namespace gs3 {
 
-constexpr int NT = 128;          // threads per 16x16 tile: two pixels each
-#ifndef FWD_UNROLL
-#define FWD_UNROLL 8
-#endif
-constexpr int kFwdUnroll = FWD_UNROLL;
-// Optional minimum blocks per SM for the forward's launch bounds
-// (0: none, the compiler's register choice).
-#ifndef FWD_MIN_BLOCKS
-#define FWD_MIN_BLOCKS 0
-#endif
-#if FWD_MIN_BLOCKS > 0
-#define FWD_BOUNDS __launch_bounds__(128, FWD_MIN_BLOCKS)
-#else
-#define FWD_BOUNDS __launch_bounds__(128)
-#endif
-#ifndef RASTER_WARP_BLOCKS
-#define RASTER_WARP_BLOCKS 1     // 1: each warp owns a compact block of the tile; 0: rows
-#endif
-
-// Pixel of lane l in warp w, pixel k of the thread (k < ppt), for a 16x16
-// tile split into 256 / (32 ppt) warps.  Blocks: a warp owns a compact
-// rectangle (8x4 for one pixel per thread, 8x8 for two, 16x8 for four or
-// more) whose pixels tend to share records and list ends; a thread's pixels
-// are vertically adjacent.  Rows: thread t owns column t % 16 of rows
-// t / 16 + k * (16 / ppt).
-__device__ __forceinline__ void tile_pixel(int tid, int ppt, int k, int &x, int &y)
-{
-    if (RASTER_WARP_BLOCKS) {
-        const int w = tid >> 5, l = tid & 31;
-        const int rw = ppt >= 4 ? 16 : 8;         // warp rectangle width
-        const int wpr = 16 / rw;                  // warps per tile row
-        const int rows = (32 / rw) * ppt;         // warp rectangle height
-        x = (w % wpr) * rw + l % rw;
-        y = (w / wpr) * rows + (l / rw) * ppt + k;
-    } else {
-        x = tid & 15;
-        y = (tid >> 4) + k * (16 / ppt);
-    }
-}
+constexpr int NT = 128;          // threads of a forward block (one 16x16 tile): two pixels each
 
 struct RasterParams {
     const float2 *mean2d;
@@ -88,25 +51,6 @@ __device__ __forceinline__ void flush_stats(unsigned long long *stats, uint32_t 
     }
 }
 
-// power of one record at the two pixels (px, py.x) and (px, py.y) of a
-// column, -0.5 (A dx^2 + C dy^2) - B dx dy, with explicit roundings so that
-// the forward and the reverse pass take bit-identical decisions; the offset
-// monomials dx^2, dx dy, dy^2 are returned for the reverse pass.  The
-// row-dependent terms go two per packed instruction.
-__device__ __forceinline__ float2 pair_power2(float2 xy, float4 co, float px, float2 py, float &dx,
-                                              float2 &dy, float &dxx, float2 &dxy, float2 &dyy)
-{
-    dx = __fsub_rn(px, xy.x);
-    dy = make_float2(__fsub_rn(py.x, xy.y), __fsub_rn(py.y, xy.y));
-    dxx = __fmul_rn(dx, dx);
-    dxy = __fmul2_rn(make_float2(dx, dx), dy);
-    dyy = __fmul2_rn(dy, dy);
-    const float axx = __fmul_rn(co.x, dxx);
-    const float2 q = __ffma2_rn(make_float2(co.z, co.z), dyy, make_float2(axx, axx));
-    const float2 nb = __fmul2_rn(make_float2(-co.y, -co.y), dxy);   // -(B dx dy), exact negation
-    return __ffma2_rn(make_float2(-0.5f, -0.5f), q, nb);
-}
-
 // The staged conic is scaled by log2(e) (scale_conic), so the power comes in
 // base-2 units and G = 2^power from one ex2.approx; alpha and dL/dpower keep
 // their natural-unit meaning.
@@ -125,10 +69,10 @@ __device__ __forceinline__ float pair_gauss(float power)
     return g;
 }
 
-// alpha >= 1/255 (Eq. 4's skip) is tested as power >= pmin on the base-2
-// power, pmin = -log2(255 o) staged with the record: forward and reverse take
-// the same decision, which differs from the test on alpha only within the
-// rounding of the exponential
+// alpha >= 1/255 (Eq. 4's skip) is tested on the base-2 power, power >=
+// -log2(255 o) staged with the record: forward and reverse take the same
+// decision, which differs from the test on alpha only within the rounding of
+// the exponential
 constexpr float kAlphaCap = 0.99f;
 constexpr float kTEps = 1e-4f;
 
@@ -164,179 +108,232 @@ __device__ __forceinline__ bool ellipse_hits_tile(float2 m, float4 co, int tx_t,
     return q <= tau;
 }
 
-// Does record o belong to tile (tx_t, ty_t)'s list (its tile rectangle holds
-// the tile; implied when bins are single tiles) and can it contribute there?
-template <bool BINNED>
-__device__ __forceinline__ bool keep_record(const RasterParams &p, int64_t o, int tx_t, int ty_t,
-                                            float2 &m, float4 &co)
+__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
+
+__device__ __forceinline__ void cp_async4(void *dst, const void *src)
 {
-    m = p.mean2d[o];
-    co = p.conic_op[o];
-    if (BINNED) {
-        int r = p.radius[o];
-        if (r <= 0) return false;
-        int x0, y0, x1, y1;
-        tile_rect(m.x, m.y, r, p.tx, p.ty, x0, y0, x1, y1);
-        if (!(tx_t >= x0 && tx_t < x1 && ty_t >= y0 && ty_t < y1)) return false;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Forward: one 16x16 tile per 128-thread block, two vertically adjacent pixels
+// a thread evaluated as a pair in packed FP32.  It is bound by instruction
+// issue (76 % of the slots, the ALU pipe busiest) where there are many tiles,
+// and by the chain of a tile's batches where there are few.  The batches
+// therefore run as a pipeline with one barrier each: while a batch of staged
+// records is composited, the next batch's candidates are in flight to
+// registers (their indices one batch earlier) and the colours of the records
+// just kept to shared memory (cp.async).  Before, each batch waited for its
+// indices, records and colours in turn, behind three barriers: 575 -> 523 us
+// at 250K Gaussians and four 1352x1014 views, 235 -> 189 us at 50K and eight
+// 480x360 views, 94 -> 67 us at 49K and one 477x363 view.  Measured slower:
+// four pixels a lane as in the reverse (676 / 272 / 95 us: it needs 120
+// registers, and fewer warps hide less), records culled per warp (576 / 204 /
+// 65 us), two candidates a thread per batch (745 / 255 / 78 us at 64
+// registers), no per-lane skip of records (548 / 223 / 78 us).
+constexpr int FWD_UNROLL = 4;
+
+struct FwdBatch {
+    float4 xyt[NT];    // mean, threshold power
+    float4 co[NT];     // conic in base-2 units, opacity
+    float4 rgbk[NT];   // colour and (bit pattern of) 1 + the list position
+};
+
+struct PixFwd2 {
+    float2 y, T, C0, C1, C2;
+    int last0, last1;
+    int alive;   // bit k: pixel k has not stopped
+    int stop;    // number of staged records up to the last stop
+};
+
+// One staged record (number `staged` of the tile's list) at the thread's two
+// pixels; a pixel takes part when its negated power is in [0, threshold] (see
+// bwd_chunk).
+template <bool STATS>
+__device__ __forceinline__ void fwd_record(PixFwd2 &P, float4 xyt, float4 co, const float4 &rgbk, float pxf, int staged,
+                                           uint32_t &n_tested, uint32_t &n_contrib)
+{
+    const uint32_t thr = __float_as_uint(xyt.z);
+    const float dx = __fsub_rn(pxf, xyt.x);
+    const float axx = __fmul_rn(co.x, __fmul_rn(dx, dx));
+    const float2 dy = __fadd2_rn(P.y, f2(-xyt.y));
+    const float2 q = __ffma2_rn(f2(co.z), __fmul2_rn(dy, dy), f2(axx));
+    const float2 np = __ffma2_rn(f2(0.5f), q, __fmul2_rn(f2(co.y), __fmul2_rn(f2(dx), dy)));
+    bool in0 = __float_as_uint(np.x) <= thr, in1 = __float_as_uint(np.y) <= thr;
+    if (STATS) n_tested += __popc(P.alive);
+    if (!(in0 || in1)) return;
+    float2 alpha = __fmul2_rn(f2(co.w), make_float2(pair_gauss(-np.x), pair_gauss(-np.y)));
+    alpha.x = fminf(kAlphaCap, in0 ? alpha.x : 0.f);
+    alpha.y = fminf(kAlphaCap, in1 ? alpha.y : 0.f);
+    float2 T = __fmul2_rn(P.T, __ffma2_rn(alpha, f2(-1.f), f2(1.f)));
+    if (fminf(T.x, T.y) < kTEps) {
+        // a pixel stops before this record (its T stays >= 1e-4 otherwise, so
+        // only a pixel that takes part can get here); its y becomes NaN, which
+        // no later record passes.  The empty asm keeps this a branch.
+        asm volatile("" ::: "memory");
+        const float nan = __int_as_float(0x7fc00000);
+        if (T.x < kTEps) {
+            alpha.x = 0.f;
+            T.x = P.T.x;
+            P.y.x = nan;
+            in0 = false;
+            P.alive &= ~1;
+        }
+        if (T.y < kTEps) {
+            alpha.y = 0.f;
+            T.y = P.T.y;
+            P.y.y = nan;
+            in1 = false;
+            P.alive &= ~2;
+        }
+        P.stop = staged;
     }
-    return ellipse_hits_tile(m, co, tx_t, ty_t);
+    const float2 w = __fmul2_rn(alpha, P.T);
+    P.C0 = __ffma2_rn(f2(rgbk.x), w, P.C0);
+    P.C1 = __ffma2_rn(f2(rgbk.y), w, P.C1);
+    P.C2 = __ffma2_rn(f2(rgbk.z), w, P.C2);
+    P.T = T;
+    const int k1 = __float_as_int(rgbk.w);
+    P.last0 = in0 ? k1 : P.last0;
+    P.last1 = in1 ? k1 : P.last1;
+    if (STATS) n_contrib += (uint32_t)in0 + (uint32_t)in1;
 }
 
-// Block-wide stream compaction, order preserving: returns this thread's slot
-// (or -1) and the number kept.
-template <int THREADS>
-__device__ __forceinline__ int compact_slot(bool keep, int *s_wcnt, int &count)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned b = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) s_wcnt[warp] = __popc(b);
-    __syncthreads();
-    int off = 0, tot = 0;
-#pragma unroll
-    for (int w = 0; w < THREADS / 32; ++w) {
-        int c = s_wcnt[w];
-        off += w < warp ? c : 0;
-        tot += c;
-    }
-    count = tot;
-    return keep ? off + __popc(b & ((1u << lane) - 1u)) : -1;
-}
-
-// Forward with two vertically adjacent pixels per thread (128 threads per
-// tile): the record loads and the column offset are shared, and the pair of
-// pixels is evaluated in packed FP32 (quadratic forms, alpha, transmittance,
-// colour), two lanes of a register pair per instruction.  The arithmetic of an
-// added pixel is the scalar one, rounding for rounding.
+// 9 blocks per SM: 54 registers without spills (8: 529 / 200 us without the
+// per-lane skip; 10: 48 registers, 562 us)
 template <bool BINNED, bool STATS>
-__global__ void FWD_BOUNDS raster_fwd2_kernel(RasterParams p)
+__global__ void __launch_bounds__(NT, 9) raster_fwd_kernel(RasterParams p)
 {
-    __shared__ float4 s_xy[NT];
-    __shared__ float4 s_co[NT];
-    __shared__ float4 s_rgbk[NT];  // colour and (bit pattern of) the list position
-    __shared__ int s_wcnt[NT / 32];
+    __shared__ FwdBatch s_batch[2];
+    __shared__ int s_wcnt[2][NT / 32];
+    __shared__ int s_count;
+    constexpr unsigned all = 0xffffffffu;
     const int tile = blockIdx.x, view = blockIdx.y;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx_t = tile % p.tx, ty_t = tile / p.tx;
-    int px, py0;
-    tile_pixel(tid, 2, 0, px, py0);
-    px += tx_t * 16;
-    py0 += ty_t * 16;
-    const bool in0 = px < p.W && py0 < p.H, in1 = px < p.W && py0 + 1 < p.H;
+    // a warp owns a compact 8x8 block, whose pixels tend to share records and list ends
+    const int px = tx_t * 16 + (warp & 1) * 8 + (lane & 7), py0 = ty_t * 16 + (warp >> 1) * 8 + (lane >> 3) * 2;
+    const bool pix0 = px < p.W && py0 < p.H, pix1 = px < p.W && py0 + 1 < p.H;
     const float pxf = (float)px + 0.5f;
-    const float2 pyf = make_float2((float)py0 + 0.5f, (float)py0 + 1.5f);
     const int binid = (ty_t / p.bin) * p.bins_x + tx_t / p.bin;
     const uint2 range = p.ranges[(int64_t)view * p.bins + binid];
     const int total = (int)(range.y - range.x);
     const int64_t vb = (int64_t)view * p.n;
-    float T[2] = {1.f, 1.f}, C0[2] = {0.f, 0.f}, C1[2] = {0.f, 0.f}, C2[2] = {0.f, 0.f};
-    int last[2] = {0, 0};
-    bool done[2] = {!in0, !in1};
+    const int64_t tg = (int64_t)view * gridDim.x + tile;   // the tile's list
+    const float nan = __int_as_float(0x7fc00000);
+    PixFwd2 P;
+    P.y = make_float2(pix0 ? (float)py0 + 0.5f : nan, pix1 ? (float)py0 + 1.5f : nan);
+    P.T = f2(1.f);
+    P.C0 = P.C1 = P.C2 = f2(0.f);
+    P.last0 = P.last1 = 0;
+    P.alive = (int)pix0 | ((int)pix1 << 1);
+    P.stop = 0;
+    if (tid == 0) s_count = 0;
     uint32_t n_tested = 0, n_contrib = 0;
-    const int64_t tg = (int64_t)view * gridDim.x + tile;  // the tile's list
-    int staged = 0;
-    // the last batch's first list index, and how far into it this thread's
-    // pixels went (all of it unless both stopped)
-    int staged_prev = 0, jlast = 0;
-    __shared__ int s_jmax;
-    if (tid == 0) s_jmax = 0;
-    for (int base = 0; base < total; base += NT) {
-        if (__syncthreads_count(done[0] && done[1]) == NT) break;
+    // the thread's candidate of the batch to be tested, and the index of the one after
+    uint32_t g = 0, g_next = 0;
+    int r;
+    float2 m;
+    float4 co;
+    auto load_index = [&](int k) { return k < total ? p.vals[range.x + k] : 0u; };
+    auto load_record = [&](int k) {
+        const bool ok = k < total;
+        r = ok ? (BINNED ? p.radius[vb + g] : 1) : 0;
+        m = ok ? p.mean2d[vb + g] : make_float2(0.f, 0.f);
+        co = ok ? p.conic_op[vb + g] : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    auto composite = [&](const FwdBatch &B, int cnt, int first) {
+        int j = 0;
+        for (; j + FWD_UNROLL <= cnt && P.alive; j += FWD_UNROLL) {
+#pragma unroll
+            for (int i = 0; i < FWD_UNROLL; ++i)
+                fwd_record<STATS>(P, B.xyt[j + i], B.co[j + i], B.rgbk[j + i], pxf, first + j + i + 1, n_tested,
+                                  n_contrib);
+        }
+        for (; j < cnt && P.alive; ++j)
+            fwd_record<STATS>(P, B.xyt[j], B.co[j], B.rgbk[j], pxf, first + j + 1, n_tested, n_contrib);
+    };
+    g = load_index(tid);
+    load_record(tid);
+    g_next = load_index(NT + tid);
+    int staged = 0, prev = 0, buf = 0;   // records staged so far, those of the batch before
+    bool open = true;
+    for (int base = 0; base < total; base += NT, buf ^= 1) {
         const int k = base + tid;
-        int64_t o = 0;
-        uint32_t g = 0;
-        bool keep = false;
-        float2 m;
-        float4 co;
-        if (k < total) {
-            g = p.vals[range.x + k];
-            o = vb + g;
-            keep = keep_record<BINNED>(p, o, tx_t, ty_t, m, co);
+        bool keep = r > 0;
+        if (BINNED && keep) {
+            int x0, y0, x1, y1;
+            tile_rect(m.x, m.y, r, p.tx, p.ty, x0, y0, x1, y1);
+            keep = tx_t >= x0 && tx_t < x1 && ty_t >= y0 && ty_t < y1;
         }
-        int cnt;
-        const int slot = compact_slot<NT>(keep, s_wcnt, cnt);
-        if (slot >= 0 && p.tl_rec && staged + slot < p.tl_cap)
-            p.tl_rec[tg * p.tl_cap + staged + slot] = make_uint2(g, (uint32_t)k);
-        staged_prev = staged;
+        keep = keep && ellipse_hits_tile(m, co, tx_t, ty_t);
+        const unsigned kept = __ballot_sync(all, keep);
+        if (lane == 0) s_wcnt[buf][warp] = __popc(kept);
+        // the barrier of the batch: its counts and the batch before's records
+        // and colours are there, and buffer `buf` (two batches ago) is free
+        cp_async_wait();
+        if (!__syncthreads_or(P.alive)) {
+            open = false;
+            break;
+        }
+        int off = 0, cnt = 0;
+#pragma unroll
+        for (int w = 0; w < NT / 32; ++w) {
+            const int c = s_wcnt[buf][w];
+            off += w < warp ? c : 0;
+            cnt += c;
+        }
+        if (keep) {
+            const int slot = off + __popc(kept & ((1u << lane) - 1u));
+            if (p.tl_rec && staged + slot < p.tl_cap)
+                p.tl_rec[tg * p.tl_cap + staged + slot] = make_uint2(g, (uint32_t)k);
+            FwdBatch &B = s_batch[buf];
+            // a threshold below 0 (the logarithm's rounding at 255 o = 1) is one no pixel passes
+            const float thr = __log2f(255.f * co.w);
+            B.xyt[slot] = make_float4(thr >= 0.f ? m.x : nan, m.y, thr, 0.f);
+            B.co[slot] = scale_conic(co);
+            float *c = &B.rgbk[slot].x;
+            const float *src = p.rgb + 3 * (vb + g);
+            cp_async4(c, src);
+            cp_async4(c + 1, src + 1);
+            cp_async4(c + 2, src + 2);
+            c[3] = __int_as_float(k + 1);
+        }
+        g = g_next;
+        load_record(k + NT);
+        g_next = load_index(k + 2 * NT);
+        composite(s_batch[buf ^ 1], prev, staged - prev);
+        prev = cnt;
         staged += cnt;
-        jlast = done[0] && done[1] ? 0 : cnt;
-        if (slot >= 0) {
-            s_xy[slot] = make_float4(m.x, m.y, -__log2f(255.f * co.w), 0.f);
-            s_co[slot] = scale_conic(co);
-            s_rgbk[slot] = make_float4(p.rgb[3 * o], p.rgb[3 * o + 1], p.rgb[3 * o + 2],
-                                       __int_as_float(k));
-        }
+    }
+    if (open) {
+        cp_async_wait();
         __syncthreads();
-#pragma unroll kFwdUnroll
-        for (int j = 0; !(done[0] && done[1]) && j < cnt; ++j) {
-            const float4 cj = s_co[j];
-            const float4 xyp = s_xy[j];
-            float dx, dxx;
-            float2 dy, dxy, dyy;
-            const float2 pw = pair_power2(make_float2(xyp.x, xyp.y), cj, pxf, pyf, dx, dy, dxx, dxy, dyy);
-            const bool t0 = !done[0] && pw.x <= 0.f && pw.x >= xyp.z;   // pixel takes part
-            const bool t1 = !done[1] && pw.y <= 0.f && pw.y >= xyp.z;
-            if (STATS) n_tested += !done[0] + !done[1];
-            if (!(t0 || t1)) continue;
-            // a pixel that does not take part has its power masked to -inf:
-            // G = 0, alpha = 0 and its transmittance stays as it is (T * 1)
-            const float g0 = pair_gauss(t0 ? pw.x : -INFINITY), g1 = pair_gauss(t1 ? pw.y : -INFINITY);
-            const float2 araw = __fmul2_rn(make_float2(cj.w, cj.w), make_float2(g0, g1));
-            float2 alpha = make_float2(fminf(kAlphaCap, araw.x), fminf(kAlphaCap, araw.y));
-            const float2 om = __ffma2_rn(alpha, make_float2(-1.f, -1.f), make_float2(1.f, 1.f));
-            const float2 Tv = make_float2(T[0], T[1]);
-            float2 tT = __fmul2_rn(Tv, om);
-            bool add0 = t0, add1 = t1;
-            if (tT.x < kTEps || tT.y < kTEps) {
-                // the pixel stops before this Gaussian (T stays >= 1e-4 otherwise,
-                // so only a pixel that takes part can get here)
-                const bool stop0 = tT.x < kTEps, stop1 = tT.y < kTEps;
-                done[0] |= stop0;
-                done[1] |= stop1;
-                add0 = add0 && !stop0;
-                add1 = add1 && !stop1;
-                if (stop0) { alpha.x = 0.f; tT.x = Tv.x; }
-                if (stop1) { alpha.y = 0.f; tT.y = Tv.y; }
-                if (done[0] && done[1]) jlast = j + 1;
-            }
-            const float2 w = __fmul2_rn(alpha, Tv);
-            const float4 ck = s_rgbk[j];
-            const float2 c0 = __ffma2_rn(make_float2(ck.x, ck.x), w, make_float2(C0[0], C0[1]));
-            const float2 c1 = __ffma2_rn(make_float2(ck.y, ck.y), w, make_float2(C1[0], C1[1]));
-            const float2 c2 = __ffma2_rn(make_float2(ck.z, ck.z), w, make_float2(C2[0], C2[1]));
-            C0[0] = c0.x; C0[1] = c0.y;
-            C1[0] = c1.x; C1[1] = c1.y;
-            C2[0] = c2.x; C2[1] = c2.y;
-            T[0] = tT.x;
-            T[1] = tT.y;
-            const int kk = __float_as_int(ck.w) + 1;
-            last[0] = add0 ? kk : last[0];
-            last[1] = add1 ? kk : last[1];
-            if (STATS) n_contrib += add0 + add1;
-        }
+        composite(s_batch[buf ^ 1], prev, staged - prev);
     }
     if (STATS) flush_stats(p.stats, n_tested, n_contrib);
     if (p.tl_rec) {
-        // records of the last batch past every thread's stop took part at no
-        // pixel (their positions are at or past every pixel's last): the list
-        // ends before them
-        if (jlast > 0) atomicMax(&s_jmax, jlast);
+        // records past every pixel's stop took part at no pixel (their
+        // positions are at or past every pixel's last): the list ends before
+        // them
+        const int mine = __reduce_max_sync(all, P.alive ? staged : P.stop);
+        if (lane == 0 && mine > 0) atomicMax(&s_count, mine);
         __syncthreads();
-        if (tid == 0) {
-            const int listed = staged_prev + s_jmax;
-            p.tl_cnt[tg] = listed <= p.tl_cap ? listed : -1;
-        }
+        if (tid == 0) p.tl_cnt[tg] = s_count <= p.tl_cap ? s_count : -1;
     }
     const int64_t HW = (int64_t)p.H * p.W;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
-        if (!(q == 0 ? in0 : in1)) continue;
+        if (!(q == 0 ? pix0 : pix1)) continue;
+        const float T = q ? P.T.y : P.T.x;
         const int64_t pix = (int64_t)(py0 + q) * p.W + px;
         float *im = p.img + (int64_t)view * 3 * HW + pix;
-        im[0] = fmaf(T[q], p.bg0, C0[q]);
-        im[HW] = fmaf(T[q], p.bg1, C1[q]);
-        im[2 * HW] = fmaf(T[q], p.bg2, C2[q]);
-        p.T_final[(int64_t)view * HW + pix] = T[q];
-        p.last[(int64_t)view * HW + pix] = last[q];
+        im[0] = fmaf(T, p.bg0, q ? P.C0.y : P.C0.x);
+        im[HW] = fmaf(T, p.bg1, q ? P.C1.y : P.C1.x);
+        im[2 * HW] = fmaf(T, p.bg2, q ? P.C2.y : P.C2.x);
+        p.T_final[(int64_t)view * HW + pix] = T;
+        p.last[(int64_t)view * HW + pix] = q ? P.last1 : P.last0;
     }
 }
 
@@ -347,8 +344,6 @@ __device__ __forceinline__ float rcp_approx(float x)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-
-__device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 
 // Reverse: one warp per 8x16 half of a tile, four vertically adjacent pixels a
 // lane as two packed pairs, no barrier anywhere; the warps of a block share
@@ -362,8 +357,8 @@ __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 //    the colour gradient) in shared memory; then lane = (record, pixels), and
 //    four lanes add up a record's 32 columns.  A shuffle butterfly per record
 //    for each pixel pair, summed over a tile's warps behind two barriers a
-//    chunk, took half of the kernel's instructions: 922 / 294 us, against
-//    664 / 203 us now.
+//    chunk, took half of the kernel's instructions: 922 / 293 us, against
+//    646 / 209 us now.
 //  - each warp keeps, of the tile's list, the records that can reach its own
 //    half (staged_hits), which the former per-tile staging could not use.
 //  - four pixels a lane share a record's loads and column offset: two pixels
@@ -807,13 +802,13 @@ extern "C" gs_status gs_raster_fwd(const gs_projected *proj, int64_t n, int V, i
     note_launch();
     cudaStream_t s = as_stream(stream);
     if (bin > 1 && p.stats)
-        raster_fwd2_kernel<true, true><<<grid, NT, 0, s>>>(p);
+        raster_fwd_kernel<true, true><<<grid, NT, 0, s>>>(p);
     else if (bin > 1)
-        raster_fwd2_kernel<true, false><<<grid, NT, 0, s>>>(p);
+        raster_fwd_kernel<true, false><<<grid, NT, 0, s>>>(p);
     else if (p.stats)
-        raster_fwd2_kernel<false, true><<<grid, NT, 0, s>>>(p);
+        raster_fwd_kernel<false, true><<<grid, NT, 0, s>>>(p);
     else
-        raster_fwd2_kernel<false, false><<<grid, NT, 0, s>>>(p);
+        raster_fwd_kernel<false, false><<<grid, NT, 0, s>>>(p);
     return launch_status("gs_raster_fwd");
 }
 
