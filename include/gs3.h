@@ -488,7 +488,7 @@ GS_API gs_status gs_viewspace_grad_accum(const float *grads, const int32_t *radi
                                          gs_stream stream);
 
 /* idx[0 .. *d_nsel) = the j < count, in increasing order, with denom[j] > 0
- * and accum[j] / denom[j] > tau (FP32).  One block; no workspace. */
+ * and accum[j] / denom[j] > tau (FP32).  One cluster of blocks; no workspace. */
 GS_API gs_status gs_select_above(const float *accum, const int32_t *denom, int64_t count, float tau,
                                  int32_t *idx, int64_t *d_nsel, gs_stream stream);
 
