@@ -1,116 +1,55 @@
 // L1 + D-SSIM loss and its gradient (Section 4.1, Eq. 6).
-// Pass 1 filters (x, y, x^2, y^2, xy) with the separable 11x11 Gaussian
+// Pass 1 filters (x, y, (x - y)^2, xy) with the separable 11x11 Gaussian
 // window, forms the SSIM map and the three per-pixel coefficients of its
 // derivative wrt (mu_x, E[x^2], E[xy]); pass 2 filters those coefficients (the
 // window is symmetric, so the adjoint is the same filter) and assembles
 // dL/dI; pass 3 reduces the block partial sums (compensated FP32).
-//
-// Both filtering passes work on 32 x 48 output tiles.  The horizontal stage
-// reads its inputs straight from global memory (through L1, as float4 where
-// rows are 16-byte aligned; in pass 1 with such rows the tile's input window
-// comes into shared memory by TMA instead) and leaves the row-filtered maps
-// in shared memory; the vertical stage filters the columns from there.  The filters use
-// the packed FP32 FMA of sm_100+ (both halves of an aligned register pair in
-// one instruction): along a row a tap pair (w_t, w_t+1) multiplies an input
-// pair (in_j, in_j+1) and the halves are added at the end; down a column the
-// two maps of a pair (x and y, x^2 and y^2, two coefficient maps) share the
-// weight.
-#include <cuda.h>
-#include <mutex>
 #include <math.h>
 
 #include "common.cuh"
-#include "tc.cuh"
 
 namespace gs3 {
 
-constexpr int SX = 32;                 // output tile width
-constexpr int SY = 48;                 // output tile height
-constexpr int LH = 5;                  // window half-width
-constexpr int SR = SY + 2 * LH;        // rows of the row-filtered maps (58)
-constexpr int HSEG = 4;                // outputs of one horizontal item
-constexpr int VSEG = 6;                // outputs of one thread in the vertical stage
+// Both filtering passes work on tiles of LX x LY outputs, columns first.  In
+// the column stage a thread walks down one of the LC = LX + 10 columns, its
+// inputs read straight from global memory (a warp's lanes on one row, so
+// coalesced at any width), and keeps LR outputs going; in the row stage a
+// thread takes LO consecutive outputs of a row of the column-filtered maps in
+// shared memory.  The passes are bound by instruction issue, so the shape is
+// chosen for the fewest instructions a pixel: the maps go through both stages
+// in pairs, in packed FP32 with one weight for both halves, as one 16-byte
+// shared-memory access a pixel; 64 columns and LR = 8 rows make 256 column
+// items, 32 rows and LO = 7 outputs make 256 row items.  A row stage whose
+// lanes stand on eight rows of an odd stride meets no bank conflict; its
+// results go through the same buffer once more to be written row by row.
+// Of the squares only (x - y)^2 is filtered: sigma_x^2 + sigma_y^2 is its
+// variance plus twice the covariance, and written so the map's numerator and
+// denominator share the covariance's rounding.
+// Four planes of three channels, 1352x1014: 277 -> 198 us for the whole call
+// (pass 1 157 -> 99 us, pass 2 109 -> 91 us, pass 3 8 -> 5 us); one 479x361
+// image 26 -> 20 us, sixteen 1920x1080 images 1 500 -> 1 060 us; the
+// gradient's error against 64 bits 6.6e-6 -> 6.1e-6 relative.  The former form
+// filtered rows first with pairs along the row (extra additions, and twice
+// the weights, fetched again at each use), staged by TMA where W is a
+// multiple of 4.  Measured and not kept: both passes on chunks of planes whose
+// coefficients stay in L2 (222 us: the chunks' last waves cost more).
+constexpr int LX = 54, LY = 32;      // outputs of a tile
+constexpr int LH = 5;                // window half-width
+constexpr int LC = LX + 2 * LH;      // columns of the column stage
+constexpr int LR = 8;                // rows of one column item
+constexpr int LO = 7;                // outputs of one row item
 constexpr int LTHREADS = 256;
-constexpr int HITEMS = SR * (SX / HSEG);
-static_assert(SX * (SY / VSEG) == LTHREADS, "vertical stage: one column segment per thread");
-static_assert(SX % HSEG == 0 && HSEG == 4, "horizontal items hold four outputs");
-
-
-// The window as tap pairs for the row filter: e[i] = (w_2i, w_2i+1) for
-// outputs whose window starts on an even input, o[i] = (w_2i-1, w_2i) with
-// w_-1 = 0 for the others.
-struct RowTaps {
-    float2 e[5], o[6];
-    float w10;
-};
-
-__device__ __forceinline__ RowTaps row_taps(const float *w)
-{
-    RowTaps t;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) t.e[i] = make_float2(w[2 * i], w[2 * i + 1]);
-    t.o[0] = make_float2(0.f, w[0]);
-#pragma unroll
-    for (int i = 1; i < 6; ++i) t.o[i] = make_float2(w[2 * i - 1], w[2 * i]);
-    t.w10 = w[10];
-    return t;
-}
-
-// Inputs of one horizontal item as pairs: m[k] = (in_2k, in_2k+1), in_j the
-// value at column B + j, B = x0 + c0 - 8 (a multiple of 4).  Output o of the
-// item (column B + 8 + o) sums in_3+o .. in_13+o.
-constexpr int NPAIR = 9;
-
-__device__ __forceinline__ void load_pairs(const float *row, int W, int B, bool vec, float2 (&m)[NPAIR])
-{
-    m[0] = make_float2(0.f, 0.f);  // in_0, in_1: never used
-    if (vec && B >= 0 && B + 16 <= W) {
-        const float4 *r4 = reinterpret_cast<const float4 *>(row + B);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const float4 v = __ldg(r4 + q);
-            m[2 * q] = make_float2(v.x, v.y);
-            m[2 * q + 1] = make_float2(v.z, v.w);
-        }
-    } else {
-#pragma unroll
-        for (int k = 1; k < 8; ++k) {
-            const int g0 = B + 2 * k, g1 = g0 + 1;
-            m[k] = make_float2(g0 >= 0 && g0 < W ? __ldg(row + g0) : 0.f,
-                               g1 >= 0 && g1 < W ? __ldg(row + g1) : 0.f);
-        }
-    }
-    const int g16 = B + 16;
-    m[8] = make_float2(g16 < W ? __ldg(row + g16) : 0.f, 0.f);
-}
-
-// Row filter of one map for the item's four outputs.
-__device__ __forceinline__ void row_filter(const float2 (&m)[NPAIR], const RowTaps &t, float (&out)[HSEG])
-{
-#pragma unroll
-    for (int o = 0; o < HSEG; o += 2) {
-        // even output o: window in_3+o .. in_13+o, pairs from in_2+o with o[]
-        float2 a = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 6; ++i) a = __ffma2_rn(t.o[i], m[1 + o / 2 + i], a);
-        out[o] = a.x + a.y;
-        // odd output o + 1: pairs from in_4+o with e[], last tap in_14+o
-        float2 b = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 5; ++i) b = __ffma2_rn(t.e[i], m[2 + o / 2 + i], b);
-        out[o + 1] = fmaf(t.w10, m[7 + o / 2].x, b.x + b.y);
-    }
-}
-
-__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+constexpr int LS = 67, LS2 = 66, LS1 = 68;   // row strides of the shared maps (float4, float2, float)
+static_assert(LC * (LY / LR) == LTHREADS, "one column item a thread");
+static_assert(LY * 8 == LTHREADS && 8 * LO >= LX && 7 * LO + LO + 2 * LH <= LS, "one row item a thread");
+static_assert(LS % 2 == 1, "eight rows meet eight bank groups");
 
 struct LossParams {
-    float win[11];        // normalised 11-tap Gaussian window (sigma 1.5), set on the host
+    float w[6];           // the normalised 11-tap Gaussian window (sigma 1.5): taps 0..5, symmetric; set on the host
     const float *x, *y;
-    int P, H, W;
+    int H, W;
     float lam;
     float invM;           // 1 / (planes H W), the mean's weight (set on the host)
-    bool vec;             // rows of x, y and the coefficient maps are 16-byte aligned
     float *ca, *cb, *cc;  // per-pixel derivative coefficients
     float2 *partial;      // [blocks]: (sum of SSIM map, sum |x - y|)
     float *d_img;
@@ -118,203 +57,145 @@ struct LossParams {
     int nblocks;
 };
 
-#ifndef SSIM_FWD_MIN_BLOCKS
-#define SSIM_FWD_MIN_BLOCKS 3  // 80 registers, no spills
-#endif
-// TMA staging of the forward's input window: columns x0 - 8 .. x0 + 39 (TW,
-// a 16-byte aligned start) and rows y0 - LH .. y0 + SY + LH - 1 of one plane
-// of each image, zero-filled outside the image by the copy itself.  Two
-// stages of TH rows, each on its own mbarrier: the row filter works through
-// the first half of the window while the second is still in flight.
-constexpr int TW = 48;
-constexpr int TH = SR / 2;   // 29 rows per stage
-static_assert(SR % 2 == 0 && TH * (SX / HSEG) <= LTHREADS, "one round of items per stage");
-constexpr uint32_t kTmaStageBytes = 2u * TH * TW * sizeof(float);   // x and y, one stage
-// each (image, stage) buffer starts on a 128-byte boundary, as the copies require
-constexpr int kTmaBufFloats = ((TH * TW * (int)sizeof(float) + 127) / 128) * 128 / (int)sizeof(float);
-constexpr uint32_t kTmaSmem = 4u * kTmaBufFloats * sizeof(float) + 128;  // + alignment slack
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
 
-template <bool TMA>
-__global__ void __launch_bounds__(LTHREADS, SSIM_FWD_MIN_BLOCKS)
-    ssim_fwd_kernel(LossParams p, const __grid_constant__ CUtensorMap tmx,
-                    const __grid_constant__ CUtensorMap tmy)
-{
-    __shared__ float2 s_xy[SR][SX];   // row-filtered (x, y)
-    __shared__ float2 s_sq[SR][SX];   // row-filtered (x^2, y^2)
-    __shared__ float s_p[SR][SX];     // row-filtered x y
-    __shared__ float red[2][LTHREADS / 32];
-    __shared__ __align__(8) unsigned long long s_mbar[2];
-    extern __shared__ __align__(128) unsigned char s_dyn[];   // TMA: [image][stage][TH][TW] floats
-    float *s_in = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(s_dyn) + 127) & ~uintptr_t(127));
-    const float *c_win = p.win;
-    const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * SX, y0 = blockIdx.y * SY, pl = blockIdx.z;
-    const int64_t HW = (int64_t)p.H * p.W;
-    const float *X = p.x + pl * HW, *Y = p.y + pl * HW;
-    float lsum = 0.f;
-    bool ok = true;
-    if (TMA) {
-        if (tid == 0) {
-            tc::mbar_init(tc::smem_u32(&s_mbar[0]), 1);
-            tc::mbar_init(tc::smem_u32(&s_mbar[1]), 1);
-        }
-        __syncthreads();
-        if (tid == 0) {
+// The six taps in registers (the empty asm keeps the compiler from fetching
+// them again at every use).
+struct Taps {
+    float w[6];
+    __device__ __forceinline__ explicit Taps(const LossParams &p)
+    {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t mbar = tc::smem_u32(&s_mbar[h]);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar),
-                             "r"(kTmaStageBytes)
-                             : "memory");
-                asm volatile(
-                    "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                    " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(tc::smem_u32(s_in + h * kTmaBufFloats)),
-                    "l"(reinterpret_cast<uint64_t>(&tmx)), "r"(x0 - 8), "r"(y0 - LH + h * TH), "r"(pl),
-                    "r"(mbar)
-                    : "memory");
-                asm volatile(
-                    "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-                    " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(tc::smem_u32(s_in + (2 + h) * kTmaBufFloats)),
-                    "l"(reinterpret_cast<uint64_t>(&tmy)), "r"(x0 - 8), "r"(y0 - LH + h * TH), "r"(pl),
-                    "r"(mbar)
-                    : "memory");
-            }
+        for (int k = 0; k < 6; ++k) {
+            w[k] = p.w[k];
+            asm volatile("" : "+f"(w[k]));
         }
     }
+    __device__ __forceinline__ float operator[](int k) const { return w[k <= 5 ? k : 10 - k]; }
+};
+
+// The order of a window's inputs, from its two ends inwards: the largest
+// weights come last for most outputs, when the sums have their size, which
+// keeps the filters' rounding error down (the gradient's 8.2e-6 -> 7.4e-6
+// relative, before (x - y)^2 took the squares' place).
+__device__ __forceinline__ constexpr int inwards(int i, int n) { return i & 1 ? n - 1 - (i >> 1) : i >> 1; }
+
+// One column item's inputs: f(k, values at input row k) for the LR + 10 rows
+// from gy0 on of column gx of N planes; 0 outside the image.  A block whose
+// whole window lies inside takes the path without tests, on 32-bit offsets.
+template <int N, typename F>
+__device__ __forceinline__ void walk_column(const float *const (&base)[N], int gx, int gy0, int H, int W, bool inside,
+                                            F &&f)
+{
+    constexpr int ROWS = LR + 2 * LH;
+    if (inside) {
+        const uint32_t step = 4u * (uint32_t)W;
+        uint32_t top = 4u * ((uint32_t)gy0 * (uint32_t)W + (uint32_t)gx), bottom = top + (ROWS - 1) * step;
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            float v[N];
+#pragma unroll
+            for (int m = 0; m < N; ++m)
+                v[m] = __ldg(reinterpret_cast<const float *>(reinterpret_cast<const char *>(base[m]) +
+                                                             (i & 1 ? bottom : top)));
+            if (i & 1) bottom -= step;
+            else top += step;
+            f(inwards(i, ROWS), v);
+        }
+    } else {
+        const bool okx = gx >= 0 && gx < W;
+        const int64_t at0 = (int64_t)gy0 * W + gx;
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            const int k = inwards(i, ROWS);
+            const bool ok = okx && gy0 + k >= 0 && gy0 + k < H;
+            float v[N];
+#pragma unroll
+            for (int m = 0; m < N; ++m) v[m] = ok ? __ldg(base[m] + at0 + (int64_t)k * W) : 0.f;
+            f(k, v);
+        }
+    }
+}
+
+// The row stage's place: a warp's lanes are eight rows x four groups of LO
+// columns.
+__device__ __forceinline__ void row_item(int &row, int &c0)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    row = (warp >> 1) * 8 + (lane & 7);
+    c0 = ((warp & 1) * 4 + (lane >> 3)) * LO;
+}
+
+template <typename I>
+__global__ void __launch_bounds__(LTHREADS, 3) ssim_fwd_kernel(LossParams p)
+{
+    __shared__ float4 s_map[LY][LS];
+    __shared__ float red[2][LTHREADS / 32];
+    const int tid = threadIdx.x;
+    const int x0 = blockIdx.x * LX, y0 = blockIdx.y * LY;
+    const int64_t HW = (int64_t)p.H * p.W;
+    const int64_t plane = (int64_t)blockIdx.z * HW;
+    const int col = tid % LC, r0 = tid / LC * LR;
+    const Taps w(p);
+    const bool inside = x0 >= LH && x0 + LX + LH <= p.W && y0 >= LH && y0 + LY + LH <= p.H && sizeof(I) == 4;
+    float lsum = 0.f;
     {
-        const RowTaps t = row_taps(c_win);
-        for (int round = 0; round < (TMA ? 2 : (HITEMS + LTHREADS - 1) / LTHREADS); ++round) {
-            int item;
-            if (TMA) {
-                // stage `round` holds rows TH round .. TH round + TH - 1; bounded
-                // wait, and a block that gives up writes NaN outputs (the loss
-                // and, through the gradient, the non-finite check report it)
-                const bool got = tc::mbar_wait(tc::smem_u32(&s_mbar[round]), 0, tc::kWaitTries);
-                ok = __syncthreads_and(ok && got);
-                if (tid >= TH * (SX / HSEG)) continue;
-                item = round * TH * (SX / HSEG) + tid;
-            } else {
-                item = round * LTHREADS + tid;
-                if (item >= HITEMS) continue;
+        const bool own = col >= LH && col < LH + LX;
+        float2 axy[LR], adp[LR];   // filtered (x, y) and ((x - y)^2, xy)
+#pragma unroll
+        for (int o = 0; o < LR; ++o) axy[o] = adp[o] = dup(0.f);
+        const float *const base[2] = {p.x + plane, p.y + plane};
+        walk_column<2>(base, x0 - LH + col, y0 + r0 - LH, p.H, p.W, inside, [&](int k, const float (&v)[2]) {
+            const float d = v[0] - v[1];
+            const float2 xy = make_float2(v[0], v[1]), dp = make_float2(d * d, v[0] * v[1]);
+            if (k >= LH && k < LH + LR) lsum += own ? fabsf(d) : 0.f;
+#pragma unroll
+            for (int o = 0; o < LR; ++o) {
+                if (k - o < 0 || k - o > 2 * LH) continue;
+                axy[o] = __ffma2_rn(dup(w[k - o]), xy, axy[o]);
+                adp[o] = __ffma2_rn(dup(w[k - o]), dp, adp[o]);
             }
-            const int r = item / (SX / HSEG), c0 = (item % (SX / HSEG)) * HSEG;
-            const int gy = y0 - LH + r;
-            float fx[HSEG], fy[HSEG], fxx[HSEG], fyy[HSEG], fxy[HSEG];
-            if (TMA || (gy >= 0 && gy < p.H)) {
-                const int B = x0 + c0 - 8;
-                float2 mx[NPAIR], my[NPAIR], mxx[NPAIR], myy[NPAIR], mxy[NPAIR];
-                if (TMA) {
-                    const int h = r / TH, rl = r - h * TH;   // stage and row within it
-                    const float2 *rx =
-                        reinterpret_cast<const float2 *>(s_in + h * kTmaBufFloats + rl * TW + c0);
-                    const float2 *ry =
-                        reinterpret_cast<const float2 *>(s_in + (2 + h) * kTmaBufFloats + rl * TW + c0);
-                    mx[0] = my[0] = make_float2(0.f, 0.f);
+        });
 #pragma unroll
-                    for (int k = 1; k < NPAIR; ++k) {
-                        mx[k] = rx[k];
-                        my[k] = ry[k];
-                    }
-                } else {
-                    load_pairs(X + (int64_t)gy * p.W, p.W, B, p.vec, mx);
-                    load_pairs(Y + (int64_t)gy * p.W, p.W, B, p.vec, my);
-                }
+        for (int o = 0; o < LR; ++o) s_map[r0 + o][col] = make_float4(axy[o].x, axy[o].y, adp[o].x, adp[o].y);
+    }
+    __syncthreads();
+    int row, c0;
+    row_item(row, c0);
+    float2 fxy[LO], fdp[LO];
 #pragma unroll
-                for (int k = 1; k < NPAIR; ++k) {
-                    mxx[k] = __fmul2_rn(mx[k], mx[k]);
-                    myy[k] = __fmul2_rn(my[k], my[k]);
-                    mxy[k] = __fmul2_rn(mx[k], my[k]);
-                }
-                row_filter(mx, t, fx);
-                row_filter(my, t, fy);
-                row_filter(mxx, t, fxx);
-                row_filter(myy, t, fyy);
-                row_filter(mxy, t, fxy);
-                // L1 term at the item's outputs in_8 .. in_11 (pairs 4 and 5)
-                if (r >= LH && r < LH + SY && gy < p.H) {
+    for (int o = 0; o < LO; ++o) fxy[o] = fdp[o] = dup(0.f);
 #pragma unroll
-                    for (int o = 0; o < HSEG; ++o) {
-                        const float2 a = mx[4 + o / 2], b = my[4 + o / 2];
-                        const float d = (o & 1) ? a.y - b.y : a.x - b.x;
-                        if (x0 + c0 + o < p.W) lsum += fabsf(d);
-                    }
-                }
-            } else {
+    for (int i = 0; i < LO + 2 * LH; ++i) {
+        const int j = inwards(i, LO + 2 * LH);
+        const float4 v = s_map[row][c0 + j];
 #pragma unroll
-                for (int o = 0; o < HSEG; ++o) fx[o] = fy[o] = fxx[o] = fyy[o] = fxy[o] = 0.f;
-            }
-#pragma unroll
-            for (int o = 0; o < HSEG; ++o) {
-                s_xy[r][c0 + o] = make_float2(fx[o], fy[o]);
-                s_sq[r][c0 + o] = make_float2(fxx[o], fyy[o]);
-                s_p[r][c0 + o] = fxy[o];
-            }
+        for (int o = 0; o < LO; ++o) {
+            if (j - o < 0 || j - o > 2 * LH) continue;
+            fxy[o] = __ffma2_rn(dup(w[j - o]), make_float2(v.x, v.y), fxy[o]);
+            fdp[o] = __ffma2_rn(dup(w[j - o]), make_float2(v.z, v.w), fdp[o]);
         }
     }
     __syncthreads();
-    // vertical: thread -> column c, rows r0 .. r0 + VSEG - 1 of the tile
-    const int c = tid % SX, r0 = (tid / SX) * VSEG;
-    float2 fxy2[VSEG], fsq2[VSEG];
-    float fp[VSEG];
-    {
-        float2 wd[11];
-#pragma unroll
-        for (int k = 0; k < 11; ++k) wd[k] = dup(c_win[k]);
-        float2 col[VSEG + 10];
-#pragma unroll
-        for (int k = 0; k < VSEG + 10; ++k) col[k] = s_xy[r0 + k][c];
-#pragma unroll
-        for (int o = 0; o < VSEG; ++o) {
-            float2 a = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int k = 0; k < 11; ++k) a = __ffma2_rn(wd[k], col[o + k], a);
-            fxy2[o] = a;
-        }
-#pragma unroll
-        for (int k = 0; k < VSEG + 10; ++k) col[k] = s_sq[r0 + k][c];
-#pragma unroll
-        for (int o = 0; o < VSEG; ++o) {
-            float2 a = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int k = 0; k < 11; ++k) a = __ffma2_rn(wd[k], col[o + k], a);
-            fsq2[o] = a;
-        }
-        float cp[VSEG + 10];
-#pragma unroll
-        for (int k = 0; k < VSEG + 10; ++k) cp[k] = s_p[r0 + k][c];
-#pragma unroll
-        for (int o = 0; o < VSEG; ++o) {
-            float a = 0.f;
-#pragma unroll
-            for (int k = 0; k < 11; ++k) a = fmaf(c_win[k], cp[o + k], a);
-            fp[o] = a;
-        }
-    }
-    // per-thread and per-warp sums in FP32 (at most VSEG * 32 terms), the
-    // block's and the final reduction in FP64
+    // per-thread and per-warp sums in FP32 (at most LO * 32 terms)
     const float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
     float ssum = 0.f;
-    const int gx = x0 + c;
+    const bool oky = y0 + row < p.H;
 #pragma unroll
-    for (int o = 0; o < VSEG; ++o) {
-        const int gy = y0 + r0 + o;
-        if (gy >= p.H || gx >= p.W) continue;
-        const float mx = fxy2[o].x, my = fxy2[o].y, exx = fsq2[o].x, eyy = fsq2[o].y, exy = fp[o];
-        const float sxx = exx - mx * mx, syy = eyy - my * my, sxy = exy - mx * my;
+    for (int o = 0; o < LO; ++o) {
+        const float mx = fxy[o].x, my = fxy[o].y;
+        const float dm = mx - my, vd = fdp[o].x - dm * dm, sxy = fdp[o].y - mx * my;
         const float n1 = 2.f * mx * my + C1, n2 = 2.f * sxy + C2;
-        const float d1 = mx * mx + my * my + C1, d2 = sxx + syy + C2;
+        // d1 = mx^2 + my^2 + C1 and d2 = sigma_x^2 + sigma_y^2 + C2
+        const float d1 = dm * dm + n1, d2 = vd + n2;
         const float idd = 1.f / (d1 * d2);
         const float sv = n1 * n2 * idd;
         // 1 / d1 = d2 idd and 1 / d2 = d1 idd
         const float ds_dmx = 2.f * my * n2 * idd - sv * 2.f * mx * (d2 * idd);
         const float ds_dsxx = -sv * (d1 * idd);
         const float ds_dsxy = 2.f * n1 * idd;
-        const int64_t oo = pl * HW + (int64_t)gy * p.W + gx;
-        const float bad = ok ? 0.f : __int_as_float(0x7fc00000);   // NaN when the copy gave up
-        p.ca[oo] = ds_dmx - 2.f * mx * ds_dsxx - my * ds_dsxy + bad;
-        p.cb[oo] = ds_dsxx + bad;
-        p.cc[oo] = ds_dsxy + bad;
-        ssum += sv + bad;
+        s_map[row][c0 + o] = make_float4(ds_dmx - 2.f * mx * ds_dsxx - my * ds_dsxy, ds_dsxx, ds_dsxy, 0.f);
+        if (oky && c0 + o < LX && x0 + c0 + o < p.W) ssum += sv;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -326,107 +207,118 @@ __global__ void __launch_bounds__(LTHREADS, SSIM_FWD_MIN_BLOCKS)
         red[1][tid >> 5] = lsum;
     }
     __syncthreads();
+    if (col < LX && x0 + col < p.W) {
+        float *ca = p.ca + plane, *cb = p.cb + plane, *cc = p.cc + plane;
+#pragma unroll
+        for (int i = 0; i < LR; ++i) {
+            const int r = tid / LC + i * (LTHREADS / LC);
+            if (y0 + r >= p.H) continue;
+            const float4 v = s_map[r][col];
+            const I at = (I)(y0 + r) * (I)p.W + (I)(x0 + col);
+            ca[at] = v.x;
+            cb[at] = v.y;
+            cc[at] = v.z;
+        }
+    }
     if (tid == 0) {
         float a = 0.f, b = 0.f;
         for (int ww = 0; ww < LTHREADS / 32; ++ww) {
             a += red[0][ww];
             b += red[1][ww];
         }
-        int64_t bid = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        p.partial[bid] = make_float2(a, b);
+        p.partial[((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = make_float2(a, b);
     }
 }
 
-#ifndef SSIM_BWD_MIN_BLOCKS
-#define SSIM_BWD_MIN_BLOCKS 4  // 62 registers, no spills
-#endif
-__global__ void __launch_bounds__(LTHREADS, SSIM_BWD_MIN_BLOCKS) ssim_bwd_kernel(LossParams p)
+template <typename I>
+__global__ void __launch_bounds__(LTHREADS, 4) ssim_bwd_kernel(LossParams p)
 {
-    __shared__ float2 s_ab[SR][SX];   // row-filtered (ca, cb)
-    __shared__ float s_c[SR][SX];     // row-filtered cc
-    const float *c_win = p.win;
+    __shared__ float2 s_ab[LY][LS2];   // filtered (ca, cb)
+    __shared__ float s_c[LY][LS1];     // filtered cc
     const int tid = threadIdx.x;
-    const int x0 = blockIdx.x * SX, y0 = blockIdx.y * SY, pl = blockIdx.z;
+    const int x0 = blockIdx.x * LX, y0 = blockIdx.y * LY;
     const int64_t HW = (int64_t)p.H * p.W;
+    const int64_t plane = (int64_t)blockIdx.z * HW;
+    const int col = tid % LC, r0 = tid / LC * LR;
+    const Taps w(p);
+    const bool inside = x0 >= LH && x0 + LX + LH <= p.W && y0 >= LH && y0 + LY + LH <= p.H && sizeof(I) == 4;
     {
-        const RowTaps t = row_taps(c_win);
-        const float *A = p.ca + pl * HW, *Bm = p.cb + pl * HW, *Cm = p.cc + pl * HW;
-        for (int item = tid; item < HITEMS; item += LTHREADS) {
-            const int r = item / (SX / HSEG), c0 = (item % (SX / HSEG)) * HSEG;
-            const int gy = y0 - LH + r;
-            float fa[HSEG], fb[HSEG], fc[HSEG];
-            if (gy >= 0 && gy < p.H) {
-                const int B = x0 + c0 - 8;
-                const int64_t ro = (int64_t)gy * p.W;
-                // all three rows in flight before any filtering
-                float2 ma[NPAIR], mb[NPAIR], mc[NPAIR];
-                load_pairs(A + ro, p.W, B, p.vec, ma);
-                load_pairs(Bm + ro, p.W, B, p.vec, mb);
-                load_pairs(Cm + ro, p.W, B, p.vec, mc);
-                row_filter(ma, t, fa);
-                row_filter(mb, t, fb);
-                row_filter(mc, t, fc);
-            } else {
+        float2 aab[LR];
+        float ac[LR];
 #pragma unroll
-                for (int o = 0; o < HSEG; ++o) fa[o] = fb[o] = fc[o] = 0.f;
-            }
+        for (int o = 0; o < LR; ++o) {
+            aab[o] = dup(0.f);
+            ac[o] = 0.f;
+        }
+        const float *const base[3] = {p.ca + plane, p.cb + plane, p.cc + plane};
+        walk_column<3>(base, x0 - LH + col, y0 + r0 - LH, p.H, p.W, inside, [&](int k, const float (&v)[3]) {
 #pragma unroll
-            for (int o = 0; o < HSEG; ++o) {
-                s_ab[r][c0 + o] = make_float2(fa[o], fb[o]);
-                s_c[r][c0 + o] = fc[o];
+            for (int o = 0; o < LR; ++o) {
+                if (k - o < 0 || k - o > 2 * LH) continue;
+                aab[o] = __ffma2_rn(dup(w[k - o]), make_float2(v[0], v[1]), aab[o]);
+                ac[o] = fmaf(w[k - o], v[2], ac[o]);
             }
+        });
+#pragma unroll
+        for (int o = 0; o < LR; ++o) {
+            s_ab[r0 + o][col] = aab[o];
+            s_c[r0 + o][col] = ac[o];
         }
     }
     __syncthreads();
-    const float invM = p.invM;
-    const int c = tid % SX, r0 = (tid / SX) * VSEG;
-    const int gx = x0 + c;
-    // the images at this thread's outputs, loaded before the column filters
-    float xv[VSEG], yv[VSEG];
-#pragma unroll
-    for (int o = 0; o < VSEG; ++o) {
-        const int gy = y0 + r0 + o;
-        const bool in = gy < p.H && gx < p.W;
-        const int64_t oo = pl * HW + (int64_t)gy * p.W + gx;
-        xv[o] = in ? __ldg(p.x + oo) : 0.f;
-        yv[o] = in ? __ldg(p.y + oo) : 0.f;
-    }
-    float2 fab[VSEG];
-    float fc[VSEG];
+    int row, c0;
+    row_item(row, c0);
     {
-        float2 wd[11];
+        float2 fab[LO];
+        float fc[LO];
 #pragma unroll
-        for (int k = 0; k < 11; ++k) wd[k] = dup(c_win[k]);
-        float2 col[VSEG + 10];
-#pragma unroll
-        for (int k = 0; k < VSEG + 10; ++k) col[k] = s_ab[r0 + k][c];
-#pragma unroll
-        for (int o = 0; o < VSEG; ++o) {
-            float2 a = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int k = 0; k < 11; ++k) a = __ffma2_rn(wd[k], col[o + k], a);
-            fab[o] = a;
+        for (int o = 0; o < LO; ++o) {
+            fab[o] = dup(0.f);
+            fc[o] = 0.f;
         }
-        float cp[VSEG + 10];
 #pragma unroll
-        for (int k = 0; k < VSEG + 10; ++k) cp[k] = s_c[r0 + k][c];
+        for (int i = 0; i < LO + 2 * LH; ++i) {
+            const int j = inwards(i, LO + 2 * LH);
+            const float2 ab = s_ab[row][c0 + j];
+            const float c = s_c[row][c0 + j];
 #pragma unroll
-        for (int o = 0; o < VSEG; ++o) {
-            float a = 0.f;
+            for (int o = 0; o < LO; ++o) {
+                if (j - o < 0 || j - o > 2 * LH) continue;
+                fab[o] = __ffma2_rn(dup(w[j - o]), ab, fab[o]);
+                fc[o] = fmaf(w[j - o], c, fc[o]);
+            }
+        }
+        __syncthreads();
 #pragma unroll
-            for (int k = 0; k < 11; ++k) a = fmaf(c_win[k], cp[o + k], a);
-            fc[o] = a;
+        for (int o = 0; o < LO; ++o) {
+            s_ab[row][c0 + o] = fab[o];
+            s_c[row][c0 + o] = fc[o];
         }
     }
+    const bool okx = col < LX && x0 + col < p.W;
+    constexpr int RSTEP = LTHREADS / LC;
+    const I first = (I)(y0 + tid / LC) * (I)p.W + (I)(x0 + col);
+    const float *X = p.x + plane, *Y = p.y + plane;
+    float *D = p.d_img + plane;
+    float xv[LR], yv[LR];
 #pragma unroll
-    for (int o = 0; o < VSEG; ++o) {
-        const int gy = y0 + r0 + o;
-        if (gy >= p.H || gx >= p.W) continue;
-        const int64_t oo = pl * HW + (int64_t)gy * p.W + gx;
-        const float diff = xv[o] - yv[o];
+    for (int i = 0; i < LR; ++i) {
+        const bool ok = okx && y0 + tid / LC + i * RSTEP < p.H;
+        const I at = first + (I)(i * RSTEP) * (I)p.W;
+        xv[i] = ok ? __ldg(X + at) : 0.f;
+        yv[i] = ok ? __ldg(Y + at) : 0.f;
+    }
+    __syncthreads();
+    if (!okx) return;
+#pragma unroll
+    for (int i = 0; i < LR; ++i) {
+        const int r = tid / LC + i * RSTEP;
+        if (y0 + r >= p.H) continue;
+        const float2 ab = s_ab[r][col];
+        const float diff = xv[i] - yv[i];
         const float sgn = diff > 0.f ? 1.f : (diff < 0.f ? -1.f : 0.f);
-        const float dssim = fab[o].x + 2.f * xv[o] * fab[o].y + yv[o] * fc[o];
-        p.d_img[oo] = ((1.f - p.lam) * sgn - p.lam * dssim) * invM;
+        const float dssim = ab.x + 2.f * xv[i] * ab.y + yv[i] * s_c[r][col];
+        D[first + (I)(i * RSTEP) * (I)p.W] = ((1.f - p.lam) * sgn - p.lam * dssim) * p.invM;
     }
 }
 
@@ -446,10 +338,19 @@ __global__ void __launch_bounds__(1024) loss_final_kernel(LossParams p)
 {
     __shared__ float red[2][32];
     float sa = 0.f, ca = 0.f, sb = 0.f, cb = 0.f;
-    for (int i = threadIdx.x; i < p.nblocks; i += blockDim.x) {
-        const float2 v = p.partial[i];
-        kahan_add(sa, ca, v.x);
-        kahan_add(sb, cb, v.y);
+    // eight loads in flight a step
+    for (int i0 = threadIdx.x; i0 < p.nblocks; i0 += 8 * blockDim.x) {
+        float2 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int i = i0 + u * (int)blockDim.x;
+            v[u] = i < p.nblocks ? p.partial[i] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            kahan_add(sa, ca, v[u].x);
+            kahan_add(sb, cb, v[u].y);
+        }
     }
     float a = sa - ca, b = sb - cb;
 #pragma unroll
@@ -481,38 +382,6 @@ __global__ void __launch_bounds__(1024) loss_final_kernel(LossParams p)
 
 static size_t a256(size_t x) { return (x + 255) & ~size_t(255); }
 
-#ifndef SSIM_TMA
-#define SSIM_TMA 1
-#endif
-
-// Tiled TMA map of a [planes][H][W] FP32 image stack with a TW x TH box.
-// False (and the L1 path is used) when the driver entry point is missing or
-// the rows are not 16-byte aligned.
-static bool make_plane_map(CUtensorMap *m, const float *base, int planes, int H, int W)
-{
-    typedef CUresult (*EncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                                    const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                    const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                    CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static EncodeTiled encode = [] {
-        void *fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                             &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            fn = nullptr;
-        return reinterpret_cast<EncodeTiled>(fn);
-    }();
-    if (!encode || W % 4 != 0 || !aligned(base, 16)) return false;
-    const cuuint64_t dims[3] = {(cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)planes};
-    const cuuint64_t strides[2] = {(cuuint64_t)W * sizeof(float), (cuuint64_t)H * W * sizeof(float)};
-    const cuuint32_t box[3] = {(cuuint32_t)TW, (cuuint32_t)TH, 1u};
-    const cuuint32_t estr[3] = {1u, 1u, 1u};
-    return encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(base), dims, strides, box,
-                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 }  // namespace gs3
 
 using namespace gs3;
@@ -521,7 +390,7 @@ extern "C" size_t gs_loss_workspace_size(int planes, int H, int W)
 {
     if (planes <= 0 || H <= 0 || W <= 0) return 0;
     size_t px = (size_t)planes * H * W;
-    size_t nb = (size_t)ceil_div(W, SX) * ceil_div(H, SY) * planes;
+    size_t nb = (size_t)ceil_div(W, LX) * ceil_div(H, LY) * planes;
     return 3 * a256(4 * px) + a256(16 * nb);
 }
 
@@ -538,44 +407,37 @@ extern "C" gs_status gs_loss_l1_dssim(const float *img, const float *target, int
     {
         double w[11], sum = 0.0;
         for (int i = 0; i < 11; ++i) sum += (w[i] = exp(-(double)((i - 5) * (i - 5)) / 4.5));
-        for (int i = 0; i < 11; ++i) p.win[i] = (float)(w[i] / sum);
+        for (int i = 0; i < 6; ++i) p.w[i] = (float)(w[i] / sum);
     }
-    p.x = img;
-    p.y = target;
-    p.P = planes;
     p.H = H;
     p.W = W;
     p.lam = lambda;
     p.invM = (float)(1.0 / ((double)planes * (double)H * (double)W));
-    size_t px = (size_t)planes * H * W;
+    const size_t px = (size_t)planes * H * W;
     char *b = reinterpret_cast<char *>(ws);
     p.ca = reinterpret_cast<float *>(b);
     p.cb = reinterpret_cast<float *>(b + a256(4 * px));
     p.cc = reinterpret_cast<float *>(b + 2 * a256(4 * px));
-    p.partial = reinterpret_cast<float2 *>(b + 3 * a256(4 * px));
-    p.d_img = d_img;
+    float2 *partial = reinterpret_cast<float2 *>(b + 3 * a256(4 * px));
     p.d_loss = d_loss;
     p.d_ssim = d_ssim;
-    p.vec = (W % 4) == 0 && aligned(img, 16) && aligned(target, 16) && aligned(ws, 16);
-    dim3 grid((unsigned)ceil_div(W, SX), (unsigned)ceil_div(H, SY), (unsigned)planes);
-    p.nblocks = (int)(grid.x * grid.y * grid.z);
+    const unsigned gx = (unsigned)ceil_div(W, LX), gy = (unsigned)ceil_div(H, LY);
+    const dim3 grid(gx, gy, (unsigned)planes);
     cudaStream_t s = as_stream(stream);
-    CUtensorMap tmx{}, tmy{};
-    const bool tma = SSIM_TMA && p.vec && make_plane_map(&tmx, img, planes, H, W) &&
-                     make_plane_map(&tmy, target, planes, H, W);
+    p.x = img;
+    p.y = target;
+    p.d_img = d_img;
+    p.partial = partial;
+    p.nblocks = (int)(gx * gy * (unsigned)planes);
+    // 32-bit offsets within a plane while its bytes fit (the 64-bit ones made
+    // the call 219 us where these make it 198)
+    const bool small = (uint64_t)H * W < (uint64_t(1) << 30);
     note_launch();
-    if (tma) {
-        static std::once_flag once;
-        std::call_once(once, [] {
-            cudaFuncSetAttribute((const void *)ssim_fwd_kernel<true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTmaSmem);
-        });
-        ssim_fwd_kernel<true><<<grid, LTHREADS, kTmaSmem, s>>>(p, tmx, tmy);
-    } else {
-        ssim_fwd_kernel<false><<<grid, LTHREADS, 0, s>>>(p, tmx, tmy);
-    }
+    if (small) ssim_fwd_kernel<uint32_t><<<grid, LTHREADS, 0, s>>>(p);
+    else ssim_fwd_kernel<int64_t><<<grid, LTHREADS, 0, s>>>(p);
     note_launch();
-    ssim_bwd_kernel<<<grid, LTHREADS, 0, s>>>(p);
+    if (small) ssim_bwd_kernel<uint32_t><<<grid, LTHREADS, 0, s>>>(p);
+    else ssim_bwd_kernel<int64_t><<<grid, LTHREADS, 0, s>>>(p);
     note_launch();
     loss_final_kernel<<<1, 1024, 0, s>>>(p);
     return launch_status("gs_loss_l1_dssim");
