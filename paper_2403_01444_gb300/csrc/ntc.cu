@@ -1,8 +1,7 @@
 // Neural Transformation Cache (Section 4.1): multi-resolution hash encoding,
-// the 32-64-64-7 MLP (FP32 SIMT path), the transformation of means and
-// rotations, the warm-up loss (Eq. 7), and the optimiser kernels (Adam,
-// non-finite check, loss-scale state).  The BF16 tensor-core MLP lives in
-// mlp_tc.cu.
+// the transformation of means and rotations, the warm-up loss (Eq. 7), and the
+// optimiser kernels (Adam, non-finite check, loss-scale state).  The
+// 32-64-64-7 MLP lives in mlp_f32.cu (FP32) and mlp_tc.cu (BF16 tensor cores).
 #include <math.h>
 #include <stdarg.h>
 #include <string.h>
@@ -194,142 +193,6 @@ __global__ void morton_kernel(const float *mean, int64_t n, GridParams g, uint32
     }
     code[i] = spread10(q[0]) | (spread10(q[1]) << 1) | (spread10(q[2]) << 2);
     idx[i] = (uint32_t)i;
-}
-
-// ------------------------------------------------------------ MLP (SIMT)
-template <typename ET>
-__global__ void __launch_bounds__(128) mlp_fwd_simt_kernel(const ET *enc, int64_t n, const float *W,
-                                                           float *raw7)
-{
-    __shared__ float sW[GS_MLP_PARAMS];
-    for (int k = threadIdx.x; k < GS_MLP_PARAMS; k += blockDim.x) sW[k] = W[k];
-    __syncthreads();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float *W1 = sW, *W2 = sW + 64 * 32, *W3 = sW + 64 * 32 + 64 * 64;
-    float x[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) x[k] = to_f32(enc[i * 32 + k]);
-    float h1[64];
-#pragma unroll
-    for (int j = 0; j < 64; ++j) {
-        float s = 0.f;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) s = fmaf(W1[j * 32 + k], x[k], s);
-        h1[j] = fmaxf(s, 0.f);
-    }
-    float o[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int j = 0; j < 64; ++j) {
-        float s = 0.f;
-#pragma unroll
-        for (int k = 0; k < 64; ++k) s = fmaf(W2[j * 64 + k], h1[k], s);
-        s = fmaxf(s, 0.f);
-#pragma unroll
-        for (int q = 0; q < 7; ++q) o[q] = fmaf(W3[q * 64 + j], s, o[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < 7; ++q) raw7[i * 7 + q] = o[q];
-}
-
-// Backward: each block owns chunks of 128 rows; per chunk every thread forms
-// its row's activations and gradients in shared memory, then every thread
-// accumulates its share of the 6592 weight gradients over the 128 rows; one
-// atomic per weight per block at the end.
-constexpr int MB_ROWS = 128;
-constexpr int MB_SX = 33, MB_SH = 65, MB_SO = 9;
-constexpr int MB_PER_THREAD = (GS_MLP_PARAMS + MB_ROWS - 1) / MB_ROWS;  // 52
-constexpr size_t MB_SMEM =
-    sizeof(float) * (GS_MLP_PARAMS + MB_ROWS * (MB_SX + 4 * MB_SH + MB_SO));
-
-template <typename ET>
-__global__ void __launch_bounds__(MB_ROWS) mlp_bwd_simt_kernel(const ET *enc, int64_t n,
-                                                               const float *W, const float *d_raw7,
-                                                               const float *d_scale, float *dW,
-                                                               float *d_enc, const uint32_t *rows,
-                                                               const int64_t *d_rows)
-{
-    extern __shared__ float smem[];
-    float *sW = smem;
-    float *sX = sW + GS_MLP_PARAMS;
-    float *sH1 = sX + MB_ROWS * MB_SX;
-    float *sH2 = sH1 + MB_ROWS * MB_SH;
-    float *sG2 = sH2 + MB_ROWS * MB_SH;
-    float *sG1 = sG2 + MB_ROWS * MB_SH;
-    float *sGO = sG1 + MB_ROWS * MB_SH;
-    for (int k = threadIdx.x; k < GS_MLP_PARAMS; k += blockDim.x) sW[k] = W[k];
-    const float *W1 = sW, *W2 = sW + 64 * 32, *W3 = sW + 64 * 32 + 64 * 64;
-    const float scale = d_scale ? *d_scale : 1.f;
-    const int t = threadIdx.x;
-    float acc[MB_PER_THREAD];
-#pragma unroll
-    for (int r = 0; r < MB_PER_THREAD; ++r) acc[r] = 0.f;
-    // with a row list, slot k of the work is row rows[k], k < *d_rows
-    const int64_t nslots = d_rows ? *d_rows : n;
-    const int64_t nchunks = (nslots + MB_ROWS - 1) / MB_ROWS;
-    __syncthreads();
-    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t k = ch * MB_ROWS + t;
-        int64_t i = k < nslots ? (rows ? (int64_t)rows[k] : k) : n;
-        bool ok = i < n;
-        float *x = sX + t * MB_SX, *h1 = sH1 + t * MB_SH, *h2 = sH2 + t * MB_SH;
-        float *g2 = sG2 + t * MB_SH, *g1 = sG1 + t * MB_SH, *go = sGO + t * MB_SO;
-        for (int k = 0; k < 32; ++k) x[k] = ok ? to_f32(enc[i * 32 + k]) : 0.f;
-        for (int j = 0; j < 64; ++j) {
-            float s = 0.f;
-            for (int k = 0; k < 32; ++k) s = fmaf(W1[j * 32 + k], x[k], s);
-            h1[j] = fmaxf(s, 0.f);
-        }
-        for (int j = 0; j < 64; ++j) {
-            float s = 0.f;
-            for (int k = 0; k < 64; ++k) s = fmaf(W2[j * 64 + k], h1[k], s);
-            h2[j] = fmaxf(s, 0.f);
-        }
-        for (int q = 0; q < 7; ++q) go[q] = ok ? d_raw7[i * 7 + q] * scale : 0.f;
-        for (int j = 0; j < 64; ++j) {
-            float s = 0.f;
-            for (int q = 0; q < 7; ++q) s = fmaf(W3[q * 64 + j], go[q], s);
-            g2[j] = h2[j] > 0.f ? s : 0.f;
-        }
-        for (int k = 0; k < 64; ++k) {
-            float s = 0.f;
-            for (int j = 0; j < 64; ++j) s = fmaf(W2[j * 64 + k], g2[j], s);
-            g1[k] = h1[k] > 0.f ? s : 0.f;
-        }
-        if (ok && d_enc) {
-            for (int m = 0; m < 32; ++m) {
-                float s = 0.f;
-                for (int k = 0; k < 64; ++k) s = fmaf(W1[k * 32 + m], g1[k], s);
-                d_enc[i * 32 + m] = s;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < MB_PER_THREAD; ++r) {
-            int e = t + r * MB_ROWS;
-            if (e < 64 * 32) {
-                int k = e >> 5, m = e & 31;
-                float s = 0.f;
-                for (int q = 0; q < MB_ROWS; ++q) s = fmaf(sG1[q * MB_SH + k], sX[q * MB_SX + m], s);
-                acc[r] += s;
-            } else if (e < 64 * 32 + 64 * 64) {
-                int e2 = e - 64 * 32, j = e2 >> 6, k = e2 & 63;
-                float s = 0.f;
-                for (int q = 0; q < MB_ROWS; ++q) s = fmaf(sG2[q * MB_SH + j], sH1[q * MB_SH + k], s);
-                acc[r] += s;
-            } else if (e < GS_MLP_PARAMS) {
-                int e3 = e - 64 * 32 - 64 * 64, o = e3 >> 6, j = e3 & 63;
-                float s = 0.f;
-                for (int q = 0; q < MB_ROWS; ++q) s = fmaf(sGO[q * MB_SO + o], sH2[q * MB_SH + j], s);
-                acc[r] += s;
-            }
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int r = 0; r < MB_PER_THREAD; ++r) {
-        int e = t + r * MB_ROWS;
-        if (e < GS_MLP_PARAMS && acc[r] != 0.f) atomicAdd(dW + e, acc[r]);
-    }
 }
 
 // ------------------------------------------------------- transformation
@@ -688,15 +551,7 @@ extern "C" gs_status ntc_mlp_fwd(const void *enc, int enc_dtype, int64_t n, cons
     GS_REQUIRE(enc && raw7, "ntc_mlp_fwd: null argument");
     if (w->precision == GS_MLP_BF16) return mlp_tc_fwd(enc, enc_dtype, n, w, raw7, as_stream(stream));
     GS_REQUIRE(w->precision == GS_MLP_FP32 && w->w_f32, "ntc_mlp_fwd: bad precision / weights");
-    int blocks = (int)ceil_div(n, 128);
-    cudaStream_t s = as_stream(stream);
-    note_launch();
-    if (enc_dtype == GS_F32)
-        mlp_fwd_simt_kernel<float><<<blocks, 128, 0, s>>>((const float *)enc, n, w->w_f32, raw7);
-    else
-        mlp_fwd_simt_kernel<__nv_bfloat16><<<blocks, 128, 0, s>>>((const __nv_bfloat16 *)enc, n, w->w_f32,
-                                                                  raw7);
-    return launch_status("ntc_mlp_fwd");
+    return mlp_f32_fwd(enc, enc_dtype, n, w, raw7, as_stream(stream));
 }
 
 extern "C" gs_status ntc_mlp_bwd(const void *enc, int enc_dtype, int64_t n, const gs_mlp *w,
@@ -711,20 +566,7 @@ extern "C" gs_status ntc_mlp_bwd(const void *enc, int enc_dtype, int64_t n, cons
     if (w->precision == GS_MLP_BF16)
         return mlp_tc_bwd(enc, enc_dtype, n, w, d_raw7, d_scale, dW, d_enc, rows, d_rows, as_stream(stream));
     GS_REQUIRE(w->precision == GS_MLP_FP32 && w->w_f32, "ntc_mlp_bwd: bad precision / weights");
-    cudaStream_t s = as_stream(stream);
-    int blocks = (int)std::min<int64_t>(ceil_div(n, MB_ROWS), 2 * num_sms());
-    if (enc_dtype == GS_F32) {
-        set_smem_limit((const void *)mlp_bwd_simt_kernel<float>, (int)MB_SMEM, s);
-        note_launch();
-        mlp_bwd_simt_kernel<float><<<blocks, MB_ROWS, MB_SMEM, s>>>((const float *)enc, n, w->w_f32,
-                                                                    d_raw7, d_scale, dW, d_enc, rows, d_rows);
-    } else {
-        set_smem_limit((const void *)mlp_bwd_simt_kernel<__nv_bfloat16>, (int)MB_SMEM, s);
-        note_launch();
-        mlp_bwd_simt_kernel<__nv_bfloat16><<<blocks, MB_ROWS, MB_SMEM, s>>>(
-            (const __nv_bfloat16 *)enc, n, w->w_f32, d_raw7, d_scale, dW, d_enc, rows, d_rows);
-    }
-    return launch_status("ntc_mlp_bwd");
+    return mlp_f32_bwd(enc, enc_dtype, n, w, d_raw7, d_scale, dW, d_enc, rows, d_rows, as_stream(stream));
 }
 
 extern "C" gs_status ntc_apply(const float *mean, const float *quat, const float *raw7, int64_t n,

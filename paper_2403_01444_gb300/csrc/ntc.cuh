@@ -111,6 +111,13 @@ struct Box {
     }
 };
 
+// FP32 MLP (mlp_f32.cu)
+gs_status mlp_f32_fwd(const void *enc, int enc_dtype, int64_t n, const gs_mlp *w, float *raw7,
+                      cudaStream_t s);
+gs_status mlp_f32_bwd(const void *enc, int enc_dtype, int64_t n, const gs_mlp *w,
+                      const float *d_raw7, const float *d_scale, float *dW, float *d_enc,
+                      const uint32_t *rows, const int64_t *d_rows, cudaStream_t s);
+
 // BF16 tensor-core MLP (mlp_tc.cu)
 gs_status mlp_tc_fwd(const void *enc, int enc_dtype, int64_t n, const gs_mlp *w, float *raw7,
                      cudaStream_t s);
