@@ -346,8 +346,8 @@ __device__ __forceinline__ float rcp_approx(float x)
 }
 
 // Reverse: one warp per 8x16 half of a tile, four vertically adjacent pixels a
-// lane as two packed pairs, no barrier anywhere; the warps of a block share
-// nothing.  What bounds it is the instruction issue of the pair arithmetic
+// lane as NP = 2 packed pairs (or 8x8 and NP = 1, see kFewTiles), no barrier
+// anywhere; the warps of a block share nothing.  What bounds it is the instruction issue of the pair arithmetic
 // and, at small images, the longest tile.  Why it is cut this way (250K
 // Gaussians, four 1352x1014 views / 50K, eight 480x360 views, one launch, by
 // CUPTI):
@@ -358,14 +358,17 @@ __device__ __forceinline__ float rcp_approx(float x)
 //    four lanes add up a record's 32 columns.  A shuffle butterfly per record
 //    for each pixel pair, summed over a tile's warps behind two barriers a
 //    chunk, took half of the kernel's instructions: 922 / 293 us, against
-//    646 / 209 us now.
+//    646 / 184 us now.
 //  - each warp keeps, of the tile's list, the records that can reach its own
 //    half (staged_hits), which the former per-tile staging could not use.
 //  - four pixels a lane share a record's loads and column offset: two pixels
-//    a lane (8x8 per warp) ran into the shared-memory pipe (79 % of its
-//    wavefronts) at 731 / 188 us.
+//    a lane (8x8 per warp) run into the shared-memory pipe (79 % of its
+//    wavefronts) where there are many tiles, 725 us against 640.
 //  - no branch on "no lane takes part": the records of a chunk run as one
 //    straight line, so that their independent parts overlap (715 -> 667 us).
+//  - with NP = 1 a batch's list entries are loaded one batch ahead, and the
+//    colours with the means instead of after the test (82 -> 76 us for 4K
+//    Gaussians in four 128x96 views; nothing to gain with NP = 2).
 //  - tiles whose list is long go first (kHeavyList).
 constexpr int BWD_WARPS = 4;                 // warps of a block (two tiles); 1, 2 and 4 measured within 2 %
 constexpr int BWD_CHUNK = 8;                 // records of a turned sum
@@ -381,10 +384,20 @@ constexpr int BWD_TEST = 128;                // records of a bin's list tested a
 // 665, 384: 212 / 685).
 constexpr int kHeavyList = 256;
 
-struct PixBwd4 {
-    int last[4];
-    float2 T[2], dC0[2], dC1[2], dC2[2], nS[2];   // nS: minus dL/dC . (colour behind)
+template <int NP>
+struct PixBwd {
+    int last[2 * NP];
+    float2 T[NP], dC0[NP], dC1[NP], dC2[NP], nS[NP];   // nS: minus dL/dC . (colour behind)
 };
+
+// Up to this many tiles per SM, in all views, a warp takes 8x8 pixels: twice
+// the warps with little more than half the instructions per record each, for
+// launches that end with a few long lists on an idle chip.  4K Gaussians, four
+// 128x96 views (192 tiles) 129 -> 76 us; 50K, eight 480x360 views (5 520) 207
+// -> 184 us; 250K, one 1352x1014 view (5 440) 154 -> 158 us; 1M, one 1920x1080
+// view (8 160) 262 -> 295 us; 250K, two 1352x1014 views (10 880) 352 -> 390 us;
+// 50K, sixteen 480x360 views (11 040) 368 -> 348 us.
+constexpr int kFewTiles = 40;
 
 struct BwdWarp {
     float4 sum4[BWD_CHUNK][BWD_ROW];   // per record and lane, over its pixels: S, S_y, S_yy, red
@@ -395,14 +408,15 @@ struct BwdWarp {
     uint2 cand[BWD_TEST + 32];         // tiles without a list: records whose rectangle holds the tile
 };
 
-// Can a staged record reach alpha >= 1/255 at some centre of the 8x16 pixels
-// from (cx, cy) on?  As ellipse_hits_tile, in the staged units (the negated
+// Can a staged record reach alpha >= 1/255 at some centre of the 8 x 8 NP
+// pixels from (cx, cy) on?  As ellipse_hits_tile, in the staged units (the negated
 // power, base 2), with the evaluation's rounding taken off the form:
 // a record dropped here is one that every pixel of the warp skips.
+template <int NP>
 __device__ __forceinline__ bool staged_hits(float4 xyt, float4 co, float cx, float cy)
 {
     const float tau = xyt.z + 0.0075f;
-    const float xa = cx - xyt.x, xb = xa + 7.f, ya = cy - xyt.y, yb = ya + 15.f;
+    const float xa = cx - xyt.x, xb = xa + 7.f, ya = cy - xyt.y, yb = ya + (8.f * NP - 1.f);
     if (xa <= 0.f && xb >= 0.f && ya <= 0.f && yb >= 0.f) return true;
     const float A = 0.5f * co.x, B = co.y, C = 0.5f * co.z;   // A dx^2 + B dx dy + C dy^2
     const float bA = 0.5f * B * __frcp_rn(A), bC = 0.5f * B * __frcp_rn(C);
@@ -447,9 +461,9 @@ __device__ __forceinline__ float2 weigh(float2 w, float2 d, float2 a)
 //   dL/dA = -S_xx / 2,  dL/dB = -S_xy,  dL/dC = -S_yy / 2,
 // S_. = sum of dL/dpower times the offsets' monomials; the sums below are of
 // -dL/dpower and of minus the weight.
-template <bool WANT_OP, bool STATS, bool GUARD>
-__device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, PixBwd4 &P, int head, int cnt, float pxf,
-                                          const float2 (&pyf)[2], float cx0, int64_t vb, uint32_t &n_tested,
+template <int NP, bool WANT_OP, bool STATS, bool GUARD>
+__device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, PixBwd<NP> &P, int head, int cnt, float pxf,
+                                          const float2 (&pyf)[NP], float cx0, int64_t vb, uint32_t &n_tested,
                                           uint32_t &n_contrib)
 {
     constexpr unsigned all = 0xffffffffu;
@@ -463,9 +477,9 @@ __device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, Pix
         const uint32_t thr = __float_as_uint(xyt.z);
         const float dx = __fsub_rn(pxf, xyt.x);
         const float axx = __fmul_rn(co.x, __fmul_rn(dx, dx));
-        float2 dy[2], dyy[2], nd[2], nw[2];
+        float2 dy[NP], dyy[NP], nd[NP], nw[NP];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < NP; ++h) {
             dy[h] = __fadd2_rn(pyf[h], f2(-xyt.y));
             dyy[h] = __fmul2_rn(dy[h], dy[h]);
             const float2 q = __ffma2_rn(f2(co.z), dyy[h], f2(axx));
@@ -497,12 +511,17 @@ __device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, Pix
                 if (!(raw.y > -kAlphaCap)) nd[h].y = 0.f;
             }
         }
-        const float2 s = __fadd2_rn(nd[0], nd[1]);
-        const float2 sy = __ffma2_rn(nd[1], dy[1], __fmul2_rn(nd[0], dy[0]));
-        const float2 syy = __ffma2_rn(nd[1], dyy[1], __fmul2_rn(nd[0], dyy[0]));
-        const float2 r = weigh<GUARD>(nw[1], P.dC0[1], weigh<GUARD>(nw[0], P.dC0[0]));
-        const float2 g = weigh<GUARD>(nw[1], P.dC1[1], weigh<GUARD>(nw[0], P.dC1[0]));
-        const float2 b = weigh<GUARD>(nw[1], P.dC2[1], weigh<GUARD>(nw[0], P.dC2[0]));
+        float2 s = nd[0], sy = __fmul2_rn(nd[0], dy[0]), syy = __fmul2_rn(nd[0], dyy[0]);
+        float2 r = weigh<GUARD>(nw[0], P.dC0[0]), g = weigh<GUARD>(nw[0], P.dC1[0]), b = weigh<GUARD>(nw[0], P.dC2[0]);
+        if (NP == 2) {
+            constexpr int q = NP - 1;
+            s = __fadd2_rn(s, nd[q]);
+            sy = __ffma2_rn(nd[q], dy[q], sy);
+            syy = __ffma2_rn(nd[q], dyy[q], syy);
+            r = weigh<GUARD>(nw[q], P.dC0[q], r);
+            g = weigh<GUARD>(nw[q], P.dC1[q], g);
+            b = weigh<GUARD>(nw[q], P.dC2[q], b);
+        }
         S.sum4[i][lane] = make_float4(s.x + s.y, sy.x + sy.y, syy.x + syy.y, r.x + r.y);
         S.sum2[i][lane] = make_float2(g.x + g.y, b.x + b.y);
     }
@@ -561,7 +580,7 @@ __device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, Pix
     __syncwarp();
 }
 
-template <bool WANT_OP, bool BINNED, bool STATS>
+template <int NP, bool WANT_OP, bool BINNED, bool STATS>
 __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams p)
 {
     __shared__ BwdWarp s_warp[BWD_WARPS];
@@ -569,7 +588,9 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
     BwdWarp &S = s_warp[threadIdx.x >> 5];
     const int view = blockIdx.y, lane = threadIdx.x & 31;
     const int unit = blockIdx.x * BWD_WARPS + (threadIdx.x >> 5);
-    const int tile = unit >> 1;
+    constexpr int UNITS = 4 / NP;   // warps of a tile
+    constexpr bool AHEAD = NP == 1;
+    const int tile = unit / UNITS, part = unit % UNITS;
     if (tile >= p.tx * p.ty) return;
     const int64_t tg = (int64_t)view * (p.tx * p.ty) + tile;
     // with the forward's list of the tile, its records are staged straight
@@ -579,20 +600,21 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
     const bool heavy = listed < 0 || listed >= kHeavyList;
     if (listed == 0 || heavy != (blockIdx.z == 0)) return;
     const int tx_t = tile % p.tx, ty_t = tile / p.tx;
-    const int wx = tx_t * 16 + (unit & 1) * 8, wy = ty_t * 16;
-    const int px = wx + (lane & 7), py0 = wy + (lane >> 3) * 4;
+    const int wx = tx_t * 16 + (part & 1) * 8, wy = ty_t * 16 + (part >> 1) * 8;
+    const int px = wx + (lane & 7), py0 = wy + (lane >> 3) * (2 * NP);
     const float cx0 = (float)wx + 0.5f, cy0 = (float)wy + 0.5f;   // centre of the warp's first pixel
     const float pxf = (float)px + 0.5f;
-    const float2 pyf[2] = {make_float2((float)py0 + 0.5f, (float)py0 + 1.5f),
-                           make_float2((float)py0 + 2.5f, (float)py0 + 3.5f)};
+    float2 pyf[NP];
+#pragma unroll
+    for (int h = 0; h < NP; ++h) pyf[h] = make_float2((float)(py0 + 2 * h) + 0.5f, (float)(py0 + 2 * h) + 1.5f);
     const int64_t vb = (int64_t)view * p.n;
     const int64_t HW = (int64_t)p.H * p.W;
-    PixBwd4 P;
+    PixBwd<NP> P;
     bool bad = false;
     {
-        float T[4], d0[4], d1[4], d2[4], ns[4];
+        float T[2 * NP], d0[2 * NP], d1[2 * NP], d2[2 * NP], ns[2 * NP];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 2 * NP; ++k) {
             const int py = py0 + k;
             P.last[k] = 0;
             T[k] = 1.f;
@@ -610,7 +632,7 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
             bad |= !isfinite(d0[k] + d1[k] + d2[k]);
         }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < NP; ++h) {
             P.T[h] = make_float2(T[2 * h], T[2 * h + 1]);
             P.dC0[h] = make_float2(d0[2 * h], d0[2 * h + 1]);
             P.dC1[h] = make_float2(d1[2 * h], d1[2 * h + 1]);
@@ -619,7 +641,7 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
         }
     }
     const bool guard = __any_sync(all, bad);
-    const int wlast = __reduce_max_sync(all, max(max(P.last[0], P.last[1]), max(P.last[2], P.last[3])));
+    const int wlast = __reduce_max_sync(all, max(max(P.last[0], P.last[1]), max(P.last[2 * NP - 2], P.last[2 * NP - 1])));
     if (wlast == 0) return;
     uint32_t n_tested = 0, n_contrib = 0;
     const uint2 *rec = p.tl_rec + tg * p.tl_cap;
@@ -631,14 +653,17 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
     int head = 0, have = 0;     // the queue: its first record's slot (a multiple of BWD_CHUNK) and its length
     int cand0 = 0, cands = 0;   // tiles without a list: the candidates not yet staged
     int left = listed >= 0 ? listed : wlast;
+    auto listed_entry = [&](int l) { return l - 1 - lane >= 0 ? rec[l - 1 - lane] : make_uint2(0u, 0x7fffffffu); };
+    uint2 e_next = make_uint2(0u, 0x7fffffffu);
+    if (AHEAD && listed >= 0) e_next = listed_entry(left);
     while (left > 0 || cands > 0 || have > 0) {
         // stage batches of 32 records, back to front, until a chunk is full
         while ((left > 0 || cands > 0) && have < BWD_CHUNK) {
             uint2 e = make_uint2(0u, 0x7fffffffu);   // (Gaussian, position)
             if (listed >= 0) {
-                const int i = left - 1 - lane;
-                if (i >= 0) e = rec[i];
+                e = AHEAD ? e_next : listed_entry(left);
                 left -= 32;
+                if (AHEAD) e_next = listed_entry(left);
             } else {
                 // a bin's list can hold tens of thousands of records, few of
                 // them this tile's: their rectangles are tested BWD_TEST at a
@@ -691,22 +716,28 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
             }
             bool keep = (int)e.y < wlast;
             float4 xyt, co;
+            float c0 = 0.f, c1 = 0.f, c2 = 0.f;
+            auto colour = [&]() {
+                const float *c = p.rgb + 3 * (vb + e.x);
+                c0 = c[0], c1 = c[1], c2 = c[2];
+            };
             if (keep) {
+                if (AHEAD) colour();
                 const float2 m = p.mean2d[vb + e.x];
                 co = p.conic_op[vb + e.x];
                 xyt = make_float4(m.x, m.y, __log2f(255.f * co.w), __uint_as_float(e.y));
                 co = scale_conic(co);
                 co.w = -co.w;
-                keep = xyt.z >= 0.f && staged_hits(xyt, co, cx0, cy0);
+                keep = xyt.z >= 0.f && staged_hits<NP>(xyt, co, cx0, cy0);
             }
             const unsigned kept = __ballot_sync(all, keep);
             if (keep) {
                 int q = head + have + __popc(kept & ((1u << lane) - 1u));
                 if (q >= BWD_QUEUE) q -= BWD_QUEUE;
-                const float *c = p.rgb + 3 * (vb + e.x);
                 S.xyt[q] = xyt;
                 S.co[q] = co;
-                S.rgbg[q] = make_float4(c[0], c[1], c[2], __uint_as_float(e.x));
+                if (!AHEAD) colour();
+                S.rgbg[q] = make_float4(c0, c1, c2, __uint_as_float(e.x));
             }
             have += __popc(kept);
         }
@@ -718,9 +749,9 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
         }
         __syncwarp();
         if (guard)
-            bwd_chunk<WANT_OP, STATS, true>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_tested, n_contrib);
+            bwd_chunk<NP, WANT_OP, STATS, true>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_tested, n_contrib);
         else
-            bwd_chunk<WANT_OP, STATS, false>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_tested, n_contrib);
+            bwd_chunk<NP, WANT_OP, STATS, false>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_tested, n_contrib);
         head += BWD_CHUNK;
         if (head == BWD_QUEUE) head = 0;
         have -= cnt;
@@ -768,16 +799,25 @@ static gs_status fill(const gs_projected *proj, int64_t n, int V, int W, int H, 
     return GS_OK;
 }
 
+template <int NP, bool WANT_OP, bool BINNED>
+static void launch_bwd(const RasterParams &p, cudaStream_t s)
+{
+    // 4 / NP warps a tile; the second layer takes the tiles with short lists
+    // (without lists every tile is the first layer's)
+    const dim3 grid((unsigned)ceil_div(4 / NP * p.tx * p.ty, BWD_WARPS), p.V, p.tl_rec ? 2 : 1);
+    if (p.stats)
+        raster_bwd_kernel<NP, WANT_OP, BINNED, true><<<grid, 32 * BWD_WARPS, 0, s>>>(p);
+    else
+        raster_bwd_kernel<NP, WANT_OP, BINNED, false><<<grid, 32 * BWD_WARPS, 0, s>>>(p);
+}
+
 template <bool WANT_OP, bool BINNED>
 static void launch_bwd(const RasterParams &p, cudaStream_t s)
 {
-    // two warps a tile; the second layer takes the tiles with short lists
-    // (without lists every tile is the first layer's)
-    const dim3 grid((unsigned)ceil_div(2 * p.tx * p.ty, BWD_WARPS), p.V, p.tl_rec ? 2 : 1);
-    if (p.stats)
-        raster_bwd_kernel<WANT_OP, BINNED, true><<<grid, 32 * BWD_WARPS, 0, s>>>(p);
+    if ((int64_t)p.tx * p.ty * p.V <= (int64_t)kFewTiles * num_sms())
+        launch_bwd<1, WANT_OP, BINNED>(p, s);
     else
-        raster_bwd_kernel<WANT_OP, BINNED, false><<<grid, 32 * BWD_WARPS, 0, s>>>(p);
+        launch_bwd<2, WANT_OP, BINNED>(p, s);
 }
 
 }  // namespace gs3
