@@ -122,6 +122,7 @@ __device__ __forceinline__ uint32_t digit_of(const SortPass &s, uint32_t k, uint
 
 __global__ void __launch_bounds__(SORT_THREADS) radix_hist_kernel(SortPass s)
 {
+    if (grid_wait()) return;
     if (byte_constant(s.kor, s.shift)) return;
     pass_buffers(s);
     __shared__ uint32_t h[RADIX];
@@ -201,6 +202,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) scan_digit_rows_kernel(uint32
                                                                       const uint32_t *kor, int shift,
                                                                       KeyBases kb)
 {
+    if (grid_wait()) return;
     if (byte_constant(kor, shift)) return;  // a radix pass that is skipped
     __shared__ uint32_t s_w[SORT_WARPS];
     __shared__ uint32_t s_carry;
@@ -280,6 +282,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 1) scan_digit_rows_kernel(uint32
 // threads store consecutive positions of each digit's run (coalesced).
 __global__ void __launch_bounds__(SORT_THREADS, 4) radix_scatter_kernel(SortPass s)
 {
+    if (grid_wait()) return;
     __shared__ uint32_t s_off[RADIX];
     __shared__ uint32_t s_tot[RADIX];
     __shared__ uint32_t s_lst[RADIX];
@@ -427,6 +430,7 @@ __global__ void __launch_bounds__(SORT_THREADS) depth_keys_kernel(const float *d
                                                                   int64_t NV, int G, uint32_t *k, uint32_t *v,
                                                                   uint32_t *hist, uint32_t *kor)
 {
+    if (grid_wait()) return;
     __shared__ uint32_t h[RADIX];
     __shared__ uint32_t s_or[2];
     h[threadIdx.x] = 0u;
@@ -863,6 +867,7 @@ __device__ __forceinline__ int cs_slot(const CsParams &p, const CsChunk &c, int 
 
 __global__ void __launch_bounds__(CS_THREADS, CS_COUNT_MIN_BLOCKS) cs_count_kernel(CsParams p)
 {
+    if (grid_wait()) return;
     extern __shared__ uint32_t s_cnt[];      // [CS_WARPS][kp / 2]: two 16-bit counters a word
     __shared__ uint8_t s_idx[CS_WARPS][32];  // lanes of the entries with pairs
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -925,6 +930,7 @@ __global__ void __launch_bounds__(CS_THREADS, CS_COUNT_MIN_BLOCKS) cs_count_kern
 
 __global__ void __launch_bounds__(CS_THREADS) cs_place_kernel(CsParams p)
 {
+    if (grid_wait()) return;
     // per key the block's first position, then per (warp, key) the running
     // offset from it
     extern __shared__ __align__(16) uint32_t s_base[];
@@ -1046,12 +1052,12 @@ static gs_status run_pass(SortPass s, cudaStream_t st, bool counts = true)
 {
     if (counts) {
         note_launch();
-        radix_hist_kernel<<<s.G, SORT_THREADS, 0, st>>>(s);
+        launch_next(radix_hist_kernel, s.G, SORT_THREADS, 0, st, s);
     }
     note_launch();
-    scan_digit_rows_kernel<<<RADIX, SORT_THREADS, 0, st>>>(s.hist, s.G, RADIX, s.kor, s.shift, KeyBases{});
+    launch_next(scan_digit_rows_kernel, RADIX, SORT_THREADS, 0, st, s.hist, s.G, RADIX, s.kor, s.shift, KeyBases{});
     note_launch();
-    radix_scatter_kernel<<<s.G, SORT_THREADS, 0, st>>>(s);
+    launch_next(radix_scatter_kernel, s.G, SORT_THREADS, 0, st, s);
     return launch_status("radix pass");
 }
 
@@ -1092,7 +1098,7 @@ static gs_status depth_sort(const float *depth, const int32_t *radius, int64_t N
     const int G = (int)std::min<int64_t>(sort_blocks(), ceil_div(NV, SORT_TILE));
     cudaMemsetAsync(w.kor, 0, 2 * sizeof(uint32_t), st);
     note_launch();
-    depth_keys_kernel<<<G, SORT_THREADS, 0, st>>>(depth, radius, NV, G, w.dk[0], w.dv[0], w.hist, w.kor);
+    launch_next(depth_keys_kernel, G, SORT_THREADS, 0, st, depth, radius, NV, G, w.dk[0], w.dv[0], w.hist, w.kor);
     cur = 0;
     for (int pass = 0; pass < 4; ++pass) {
         SortPass s{};
@@ -1164,12 +1170,12 @@ static gs_status count_sort_views(const gs_projected *proj, int64_t n, int v0, i
     set_smem_limit((const void *)cs_count_kernel, smem_count, st);
     set_smem_limit((const void *)cs_place_kernel, smem_place, st);
     note_launch();
-    cs_count_kernel<<<G, CS_THREADS, smem_count, st>>>(cp);
+    launch_next(cs_count_kernel, G, CS_THREADS, smem_count, st, cp);
     note_launch();
     const KeyBases kb{w.done, capacity, d_count, w.n_eff, d_err, ranges + 2 * (int64_t)v0 * bins, v0 > 0};
-    scan_digit_rows_kernel<<<nkeys, SORT_THREADS, 0, st>>>(w.hist, G, nkeys, nullptr, 0, kb);
+    launch_next(scan_digit_rows_kernel, nkeys, SORT_THREADS, 0, st, w.hist, G, nkeys, nullptr, 0, kb);
     note_launch();
-    cs_place_kernel<<<G, CS_THREADS, smem_place, st>>>(cp);
+    launch_next(cs_place_kernel, G, CS_THREADS, smem_place, st, cp);
     return launch_status("gs_bin_sort");
 }
 

@@ -129,6 +129,7 @@ __device__ __forceinline__ void row_item(int &row, int &c0)
 template <typename I>
 __global__ void __launch_bounds__(LTHREADS, 3) ssim_fwd_kernel(LossParams p)
 {
+    if (grid_wait()) return;
     __shared__ float4 s_map[LY][LS];
     __shared__ float red[2][LTHREADS / 32];
     const int tid = threadIdx.x;
@@ -233,6 +234,7 @@ __global__ void __launch_bounds__(LTHREADS, 3) ssim_fwd_kernel(LossParams p)
 template <typename I>
 __global__ void __launch_bounds__(LTHREADS, 4) ssim_bwd_kernel(LossParams p)
 {
+    if (grid_wait()) return;
     __shared__ float2 s_ab[LY][LS2];   // filtered (ca, cb)
     __shared__ float s_c[LY][LS1];     // filtered cc
     const int tid = threadIdx.x;
@@ -336,6 +338,7 @@ __device__ __forceinline__ void kahan_add(float &s, float &c, float x)
 // the 1024 shares added in a tree (error about log2(1024) roundings).
 __global__ void __launch_bounds__(1024) loss_final_kernel(LossParams p)
 {
+    if (grid_wait()) return;
     __shared__ float red[2][32];
     float sa = 0.f, ca = 0.f, sb = 0.f, cb = 0.f;
     // eight loads in flight a step
@@ -433,12 +436,12 @@ extern "C" gs_status gs_loss_l1_dssim(const float *img, const float *target, int
     // the call 219 us where these make it 198)
     const bool small = (uint64_t)H * W < (uint64_t(1) << 30);
     note_launch();
-    if (small) ssim_fwd_kernel<uint32_t><<<grid, LTHREADS, 0, s>>>(p);
-    else ssim_fwd_kernel<int64_t><<<grid, LTHREADS, 0, s>>>(p);
+    if (small) launch_next(ssim_fwd_kernel<uint32_t>, grid, LTHREADS, 0, s, p);
+    else launch_next(ssim_fwd_kernel<int64_t>, grid, LTHREADS, 0, s, p);
     note_launch();
-    if (small) ssim_bwd_kernel<uint32_t><<<grid, LTHREADS, 0, s>>>(p);
-    else ssim_bwd_kernel<int64_t><<<grid, LTHREADS, 0, s>>>(p);
+    if (small) launch_next(ssim_bwd_kernel<uint32_t>, grid, LTHREADS, 0, s, p);
+    else launch_next(ssim_bwd_kernel<int64_t>, grid, LTHREADS, 0, s, p);
     note_launch();
-    loss_final_kernel<<<1, 1024, 0, s>>>(p);
+    launch_next(loss_final_kernel, 1, 1024, 0, s, p);
     return launch_status("gs_loss_l1_dssim");
 }

@@ -287,6 +287,7 @@ __global__ void __launch_bounds__(256) warmup_kernel(const float *raw7, int64_t 
 // (g 16-byte aligned); block 0 also takes the scalar tail.
 __global__ void __launch_bounds__(256) check_finite_kernel(const float *g, int64_t n, gs_train_state *st)
 {
+    if (grid_wait()) return;
     const int64_t n4 = n / 4;
     const float4 *g4 = reinterpret_cast<const float4 *>(g);
     const int64_t q0 = (int64_t)blockIdx.x * blockDim.x * 4 + threadIdx.x;
@@ -349,6 +350,7 @@ __global__ void ADAM_BOUNDS adam_kernel(float *__restrict__ p, float *__restrict
                                                    const gs_train_state *__restrict__ st,
                                                    void *__restrict__ shadow)
 {
+    if (grid_wait()) return;
     const bool skip = st->found_inf != 0;
     // bias corrections 1 - b^t as -expm1(t log b): no cancellation when b is close to 1
     const int t = st->step + 1;
@@ -411,6 +413,7 @@ __global__ void ADAM_BOUNDS adam_kernel(float *__restrict__ p, float *__restrict
 
 __global__ void state_advance_kernel(gs_train_state *st, int growth)
 {
+    if (grid_wait()) return;
     if (st->found_inf) {
         st->loss_scale *= 0.5f;
         st->clean_steps = 0;
@@ -622,7 +625,7 @@ extern "C" gs_status gs_check_finite(const float *g, int64_t n, gs_train_state *
     GS_REQUIRE(aligned(g, 16), "gs_check_finite: g must be 16-byte aligned");
     const int blocks = (int)std::max<int64_t>(ceil_div(n / 4, 256 * 4), 1);
     note_launch();
-    check_finite_kernel<<<blocks, 256, 0, as_stream(stream)>>>(g, n, d_state);
+    launch_next(check_finite_kernel, blocks, 256, 0, as_stream(stream), g, n, d_state);
     return launch_status("gs_check_finite");
 }
 
@@ -644,11 +647,11 @@ extern "C" gs_status adam_step(float *p, float *g, float *m, float *v, int64_t n
     cudaStream_t s = as_stream(stream);
     note_launch();
     if (!shadow)
-        adam_kernel<GS_NONE><<<blocks, 256, 0, s>>>(p, g, m, v, n, *hp, d_state, nullptr);
+        launch_next(adam_kernel<GS_NONE>, blocks, 256, 0, s, p, g, m, v, n, *hp, d_state, nullptr);
     else if (shadow_dtype == GS_F16)
-        adam_kernel<GS_F16><<<blocks, 256, 0, s>>>(p, g, m, v, n, *hp, d_state, shadow);
+        launch_next(adam_kernel<GS_F16>, blocks, 256, 0, s, p, g, m, v, n, *hp, d_state, shadow);
     else
-        adam_kernel<GS_BF16><<<blocks, 256, 0, s>>>(p, g, m, v, n, *hp, d_state, shadow);
+        launch_next(adam_kernel<GS_BF16>, blocks, 256, 0, s, p, g, m, v, n, *hp, d_state, shadow);
     return launch_status("adam_step");
 }
 
@@ -657,6 +660,6 @@ extern "C" gs_status gs_train_state_advance(gs_train_state *d_state, int growth_
 {
     GS_REQUIRE(d_state, "gs_train_state_advance: null state");
     note_launch();
-    state_advance_kernel<<<1, 1, 0, as_stream(stream)>>>(d_state, growth_interval);
+    launch_next(state_advance_kernel, 1, 1, 0, as_stream(stream), d_state, growth_interval);
     return launch_status("gs_train_state_advance");
 }

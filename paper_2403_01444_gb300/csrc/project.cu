@@ -257,6 +257,7 @@ __device__ __forceinline__ void load_sh(const ProjectParams &p, int64_t i, float
 template <int DEG>
 __global__ void __launch_bounds__(256, PROJ_FWD_MIN_BLOCKS) project_fwd_kernel(ProjectParams p)
 {
+    if (grid_wait()) return;
     constexpr int K = (DEG + 1) * (DEG + 1);
     extern __shared__ gs_camera s_cams[];
     for (int k = threadIdx.x; k < p.V; k += blockDim.x) s_cams[k] = p.cams[k];
@@ -442,6 +443,7 @@ __device__ __forceinline__ void bwd_finish(const ProjectParams &p, const GaussLo
 template <bool FULL, int DEG>
 __global__ void __launch_bounds__(128) project_bwd_kernel(ProjectParams p)
 {
+    if (grid_wait()) return;
     constexpr int K = (DEG + 1) * (DEG + 1);
     extern __shared__ gs_camera s_cams[];
     for (int k = threadIdx.x; k < p.V; k += blockDim.x) s_cams[k] = p.cams[k];
@@ -500,6 +502,7 @@ __global__ void __launch_bounds__(128) project_bwd_kernel(ProjectParams p)
 template <bool FULL, int DEG, int VP>
 __global__ void __launch_bounds__(128) project_bwd_views_kernel(ProjectParams p)
 {
+    if (grid_wait()) return;
     constexpr int K = (DEG + 1) * (DEG + 1);
     extern __shared__ gs_camera s_cams[];
     for (int k = threadIdx.x; k < p.V; k += blockDim.x) s_cams[k] = p.cams[k];
@@ -583,7 +586,7 @@ static void launch_bwd_views(const ProjectParams &p, size_t shm, cudaStream_t s)
     auto go = [&](auto vp) {
         constexpr int VP = decltype(vp)::value;
         const int blocks = (int)ceil_div((FULL ? p.count : p.n) * VP, threads);
-        project_bwd_views_kernel<FULL, DEG, VP><<<blocks, threads, shm, s>>>(p);
+        launch_next(project_bwd_views_kernel<FULL, DEG, VP>, blocks, threads, shm, s, p);
     };
     if (p.V <= 1) go(std::integral_constant<int, 1>());
     else if (p.V <= 2) go(std::integral_constant<int, 2>());
@@ -610,10 +613,10 @@ static void launch_bwd(const ProjectParams &p, cudaStream_t s)
     }
     const int blocks = (int)ceil_div(FULL ? p.count : p.n, threads);
     switch (p.deg) {
-    case 0: project_bwd_kernel<FULL, 0><<<blocks, threads, shm, s>>>(p); break;
-    case 1: project_bwd_kernel<FULL, 1><<<blocks, threads, shm, s>>>(p); break;
-    case 2: project_bwd_kernel<FULL, 2><<<blocks, threads, shm, s>>>(p); break;
-    default: project_bwd_kernel<FULL, 3><<<blocks, threads, shm, s>>>(p); break;
+    case 0: launch_next(project_bwd_kernel<FULL, 0>, blocks, threads, shm, s, p); break;
+    case 1: launch_next(project_bwd_kernel<FULL, 1>, blocks, threads, shm, s, p); break;
+    case 2: launch_next(project_bwd_kernel<FULL, 2>, blocks, threads, shm, s, p); break;
+    default: launch_next(project_bwd_kernel<FULL, 3>, blocks, threads, shm, s, p); break;
     }
 }
 
@@ -673,10 +676,10 @@ extern "C" gs_status gs_project(const gs_gaussians *g, const gs_camera *d_cams, 
     const size_t shm = sizeof(gs_camera) * V;
     cudaStream_t s = as_stream(stream);
     switch (p.deg) {
-    case 0: project_fwd_kernel<0><<<blocks, threads, shm, s>>>(p); break;
-    case 1: project_fwd_kernel<1><<<blocks, threads, shm, s>>>(p); break;
-    case 2: project_fwd_kernel<2><<<blocks, threads, shm, s>>>(p); break;
-    default: project_fwd_kernel<3><<<blocks, threads, shm, s>>>(p); break;
+    case 0: launch_next(project_fwd_kernel<0>, blocks, threads, shm, s, p); break;
+    case 1: launch_next(project_fwd_kernel<1>, blocks, threads, shm, s, p); break;
+    case 2: launch_next(project_fwd_kernel<2>, blocks, threads, shm, s, p); break;
+    default: launch_next(project_fwd_kernel<3>, blocks, threads, shm, s, p); break;
     }
     return launch_status("gs_project");
 }

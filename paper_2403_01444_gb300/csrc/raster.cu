@@ -205,6 +205,7 @@ __device__ __forceinline__ void fwd_record(PixFwd2 &P, float4 xyt, float4 co, co
 template <bool BINNED, bool STATS>
 __global__ void __launch_bounds__(NT, 9) raster_fwd_kernel(RasterParams p)
 {
+    if (grid_wait()) return;
     __shared__ FwdBatch s_batch[2];
     __shared__ int s_wcnt[2][NT / 32];
     __shared__ int s_count;
@@ -583,6 +584,7 @@ __device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, Pix
 template <int NP, bool WANT_OP, bool BINNED, bool STATS>
 __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams p)
 {
+    if (grid_wait()) return;
     __shared__ BwdWarp s_warp[BWD_WARPS];
     constexpr unsigned all = 0xffffffffu;
     BwdWarp &S = s_warp[threadIdx.x >> 5];
@@ -806,9 +808,9 @@ static void launch_bwd(const RasterParams &p, cudaStream_t s)
     // (without lists every tile is the first layer's)
     const dim3 grid((unsigned)ceil_div(4 / NP * p.tx * p.ty, BWD_WARPS), p.V, p.tl_rec ? 2 : 1);
     if (p.stats)
-        raster_bwd_kernel<NP, WANT_OP, BINNED, true><<<grid, 32 * BWD_WARPS, 0, s>>>(p);
+        launch_next(raster_bwd_kernel<NP, WANT_OP, BINNED, true>, grid, 32 * BWD_WARPS, 0, s, p);
     else
-        raster_bwd_kernel<NP, WANT_OP, BINNED, false><<<grid, 32 * BWD_WARPS, 0, s>>>(p);
+        launch_next(raster_bwd_kernel<NP, WANT_OP, BINNED, false>, grid, 32 * BWD_WARPS, 0, s, p);
 }
 
 template <bool WANT_OP, bool BINNED>
@@ -842,13 +844,13 @@ extern "C" gs_status gs_raster_fwd(const gs_projected *proj, int64_t n, int V, i
     note_launch();
     cudaStream_t s = as_stream(stream);
     if (bin > 1 && p.stats)
-        raster_fwd_kernel<true, true><<<grid, NT, 0, s>>>(p);
+        launch_next(raster_fwd_kernel<true, true>, grid, NT, 0, s, p);
     else if (bin > 1)
-        raster_fwd_kernel<true, false><<<grid, NT, 0, s>>>(p);
+        launch_next(raster_fwd_kernel<true, false>, grid, NT, 0, s, p);
     else if (p.stats)
-        raster_fwd_kernel<false, true><<<grid, NT, 0, s>>>(p);
+        launch_next(raster_fwd_kernel<false, true>, grid, NT, 0, s, p);
     else
-        raster_fwd_kernel<false, false><<<grid, NT, 0, s>>>(p);
+        launch_next(raster_fwd_kernel<false, false>, grid, NT, 0, s, p);
     return launch_status("gs_raster_fwd");
 }
 
