@@ -62,7 +62,7 @@ class NTCTransform(torch.autograd.Function):
         quat_t = torch.empty(n, 4, device=dev)
         gs3.ntc_encode_fwd(mean, n, c.grid, table_in, enc)
         gs3.ntc_mlp_fwd(enc, n, mlp, raw7)
-        gs3.ntc_apply(mean, quat, raw7, n, c.aabb, c.order, mean_t, quat_t)
+        gs3.ntc_apply(mean, quat, raw7, n, c.grid.aabb, c.order, mean_t, quat_t)
         ctx.c, ctx.mlp, ctx.table_shape = c, mlp, table.shape
         ctx.save_for_backward(mean, quat, enc, raw7)
         return mean_t, quat_t
@@ -74,7 +74,7 @@ class NTCTransform(torch.autograd.Function):
         d_mean_t = torch.zeros(n, 3, device=dev) if d_mean_t is None else d_mean_t.contiguous()
         d_quat_t = torch.zeros(n, 4, device=dev) if d_quat_t is None else d_quat_t.contiguous()
         d_raw7 = torch.empty(n, 7, device=dev)
-        gs3.ntc_apply_bwd(mean, quat, raw7, n, c.aabb, c.order, d_mean_t, d_quat_t, d_raw7)
+        gs3.ntc_apply_bwd(mean, quat, raw7, n, c.grid.aabb, c.order, d_mean_t, d_quat_t, d_raw7)
         d_w = torch.zeros(gs3.MLP_PARAMS, device=dev)
         d_enc = torch.empty(n, 32, device=dev)
         gs3.ntc_mlp_bwd(enc, n, ctx.mlp, d_raw7, None, d_w, d_enc)
