@@ -711,7 +711,15 @@ constexpr int CS_MAX_ENTRIES = 4095;     // entries per warp at most: CS_WARPS x
 // one by one (bins of 2x2 tiles), 500K Gaussians 1 151 -> 819 us, 100K 303 ->
 // 500 us.
 constexpr int64_t CS_GROUP_ENTRIES = 400000;
-constexpr int CS_BLOCKS_PER_SM = 4;
+// Blocks of the counting sort's grid per SM, three of which are resident: the
+// resident blocks write into every list at once, each at its own depths, a few
+// pairs per list and warp, and the sectors stay in L2 until they are whole only
+// if that window is well below the 129 MB of L2.  Placing 48M pairs into 2 040
+// lists (four of sixteen 1920x1080 views, 1M Gaussians) in 3 / 4 / 6 / 9 / 12 /
+// 18 blocks an SM: 868 / 589 / 419 / 402 / 405 / 403 us, counting 143 / 142 /
+// 136 / 142 / 160 / 188 us; four 1352x1014 views of 250K, where
+// CS_MIN_ENTRIES bounds the grid at 6.4: 37 + 74 us with 4, 36 + 72 with 9.
+constexpr int CS_BLOCKS_PER_SM = 9;
 constexpr int CS_COUNT_MIN_BLOCKS = 3;   // count kernel: 42 registers, room for its loads run ahead
 
 // Keys padded to a multiple of 8, so a warp's 16-bit row is whole 16-byte words.
