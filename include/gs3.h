@@ -305,8 +305,8 @@ GS_API gs_status gs_raster_fwd(const gs_projected *proj, int64_t n, int V, int W
 
 /* Reverse of gs_raster_fwd: walks each pixel's list back to front from
  * `last`, recomputing T_i = T_{i+1} / (1 - alpha_i) from T_final (no per-pair
- * state is stored).  Per-(view, Gaussian) gradients are reduced across each
- * warp and each tile before one vector atomic per (Gaussian, tile).
+ * state is stored).  Per-(view, Gaussian) gradients are summed over each
+ * warp's pixels (a half or a quarter of a tile) before the FP32 atomics.
  * Overwrites grads[V][N][8] = dL/d(u, v, A, B, C, r, g, b) and, when non-NULL,
  * d_opacity[V][N].  bg is a host array of 3 floats.  d_stats (device
  * uint64[2], or NULL) accumulates the pairs walked and the pairs that had
