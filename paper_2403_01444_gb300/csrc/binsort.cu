@@ -10,7 +10,8 @@
 //      of the keys and of their complements; before the counting sort, a
 //      pass on a byte that is the same in every key is skipped whole and the
 //      kernels of each pass find the buffer holding the keys from the parity
-//      of the passes before it that ran (elsewhere such a pass is a copy);
+//      of the passes before it that ran (elsewhere such a pass is a copy).  Up
+//      to DC_MAX_ENTRIES entries one cluster of blocks does all of it;
 //   2. the pairs of every entry's bins are ordered on the (view * bins + bin)
 //      key alone, stably, so each list keeps its entries' depth order.  When
 //      the per-warp key tables fit in shared memory (V * bins <= CS_MAX_KEYS)
@@ -28,6 +29,8 @@
 // scatter): no inter-block waits, deterministic output.  Equal digits or
 // keys within a warp are found with one ballot per bit (ballot_match), which
 // measured faster here than __match_any_sync.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -1003,6 +1006,174 @@ __global__ void __launch_bounds__(CS_THREADS) cs_place_kernel(CsParams p)
     }
 }
 
+// Few entries: the whole depth sort by one cluster of eight blocks.  The radix
+// passes above are thirteen launches of two to five microseconds each, however
+// few the entries; here a pass is two cluster barriers.  Warp w of block b
+// owns R x 32 consecutive entries, a register each a round: their ranks among
+// the warp's equal digits come from ballots and the warp's own row of
+// counters, the rows are scanned over the block's warps, and the blocks'
+// digit totals are read through distributed shared memory.  Entries pass
+// between the blocks through the sort's global buffers (L2).  The same
+// order, the same skipped bytes and the same buffers as the passes above.
+// What bounds it is the chain of a warp's rounds (about 1.4 us a round and
+// pass), so the limit is where the passes above catch up.  Whole binning, this
+// way against the launches, in a graph / in a stream: 1K entries 30 against 47 /
+// 30 against 48 us, 16K 38 / 51 and 39 / 68, 32K 49 / 53 and 50 / 71, 40K 55 /
+// 53 and 56 / 73, 64K 71 / 53 and 74 / 75.
+constexpr int DC_CTAS = 8, DC_THREADS = 1024, DC_WARPS = DC_THREADS / 32, DC_ROUNDS = 4;
+constexpr int DC_ROW = RADIX + 1;   // a digit's counters of 8 w rows meet different banks
+constexpr int64_t DC_MAX_ENTRIES = (int64_t)DC_CTAS * DC_THREADS * DC_ROUNDS;   // 32 768
+
+__global__ void __cluster_dims__(DC_CTAS, 1, 1) __launch_bounds__(DC_THREADS)
+    depth_sort_cluster_kernel(const float *depth, const int32_t *radius, int NV, uint32_t *k0, uint32_t *k1,
+                              uint32_t *v0, uint32_t *v1, uint32_t *kor)
+{
+    if (grid_wait()) return;
+    namespace cg = cooperative_groups;
+    __shared__ uint32_t s_cnt[DC_WARPS][DC_ROW];   // ranks so far, then the warps before
+    __shared__ uint32_t s_tot[RADIX], s_base[RADIX];
+    __shared__ uint32_t s_or[2], s_scan[RADIX / 32];
+    constexpr unsigned all = 0xffffffffu;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = (int)cluster.block_rank();
+    const int R = (NV + DC_CTAS * DC_THREADS - 1) / (DC_CTAS * DC_THREADS);   // <= DC_ROUNDS
+    const int e0 = (rank * DC_WARPS + warp) * R * 32 + lane;
+    uint32_t key[DC_ROUNDS], val[DC_ROUNDS];
+    uint32_t o1 = 0u, o0 = 0u;
+    if (tid < 2) s_or[tid] = 0u;
+#pragma unroll
+    for (int r = 0; r < DC_ROUNDS; ++r) {
+        const int e = e0 + 32 * r;
+        key[r] = 0u;
+        val[r] = (uint32_t)e;
+        if (r < R && e < NV) {
+            key[r] = radius[e] > 0 ? __float_as_uint(depth[e]) : 0xffffffffu;
+            o1 |= key[r];
+            o0 |= ~key[r];
+        }
+    }
+    o1 = __reduce_or_sync(all, o1);
+    o0 = __reduce_or_sync(all, o0);
+    __syncthreads();
+    if (lane == 0) {
+        atomicOr(&s_or[0], o1);
+        atomicOr(&s_or[1], o0);
+    }
+    cluster.sync();
+    o1 = o0 = 0u;
+#pragma unroll
+    for (int c = 0; c < DC_CTAS; ++c) {
+        const uint32_t *r = cluster.map_shared_rank(s_or, c);
+        o1 |= r[0];
+        o0 |= r[1];
+    }
+    const uint32_t diff = o1 & o0;
+    if (rank == 0 && tid == 0) {
+        kor[0] = o1;
+        kor[1] = o0;
+    }
+    bool first = true;
+    int cur = 0;
+    for (int shift = 0; shift < 32; shift += 8) {
+        if (((diff >> shift) & (RADIX - 1)) == 0u) continue;
+        if (!first) {
+            const uint32_t *kin = cur ? k1 : k0, *vin = cur ? v1 : v0;
+#pragma unroll
+            for (int r = 0; r < DC_ROUNDS; ++r) {
+                const int e = e0 + 32 * r;
+                if (r < R && e < NV) {
+                    key[r] = __ldcg(kin + e);
+                    val[r] = __ldcg(vin + e);
+                }
+            }
+        }
+        first = false;
+        uint32_t *cnt = s_cnt[warp];
+        for (int d = lane; d < RADIX; d += 32) cnt[d] = 0u;
+        __syncwarp();
+        uint32_t place[DC_ROUNDS];
+#pragma unroll
+        for (int r = 0; r < DC_ROUNDS; ++r) {
+            if (r >= R) break;
+            const bool ok = e0 + 32 * r < NV;
+            const uint32_t d = (key[r] >> shift) & (RADIX - 1);
+            const unsigned peers = ballot_match<8>(d, ok);
+            const uint32_t before = ok ? cnt[d] : 0u;
+            place[r] = before + __popc(peers & ((1u << lane) - 1u));
+            __syncwarp();
+            if (ok && lane == __ffs(peers) - 1) cnt[d] = before + __popc(peers);
+            __syncwarp();
+        }
+        __syncthreads();
+        {   // four threads a digit, eight warps each
+            const int d = tid >> 2, w0 = (tid & 3) * 8;
+            uint32_t x[8], sum = 0u;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                x[w] = s_cnt[w0 + w][d];
+                sum += x[w];
+            }
+            uint32_t inc = sum;
+#pragma unroll
+            for (int o = 1; o < 4; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(all, inc, o, 4);
+                if ((tid & 3) >= o) inc += y;
+            }
+            uint32_t run = inc - sum;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                s_cnt[w0 + w][d] = run;
+                run += x[w];
+            }
+            if ((tid & 3) == 3) s_tot[d] = inc;
+        }
+        cluster.sync();
+        uint32_t total = 0u, before = 0u, inc = 0u;
+        if (tid < RADIX) {
+#pragma unroll
+            for (int c = 0; c < DC_CTAS; ++c) {
+                const uint32_t t = cluster.map_shared_rank(s_tot, c)[tid];
+                before += c < rank ? t : 0u;
+                total += t;
+            }
+            inc = total;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(all, inc, o);
+                if (lane >= o) inc += y;
+            }
+            if (lane == 31) s_scan[warp] = inc;
+        }
+        __syncthreads();
+        if (tid < RADIX) {
+            uint32_t lower = inc - total;
+#pragma unroll
+            for (int w = 0; w < RADIX / 32; ++w) lower += w < warp ? s_scan[w] : 0u;
+            s_base[tid] = lower + before;
+        }
+        __syncthreads();
+        const bool last = (diff >> shift >> 8) == 0u;   // the placement after this reads the values only
+        uint32_t *kout = cur ? k0 : k1, *vout = cur ? v0 : v1;
+#pragma unroll
+        for (int r = 0; r < DC_ROUNDS; ++r) {
+            if (r >= R || e0 + 32 * r >= NV) continue;
+            const uint32_t d = (key[r] >> shift) & (RADIX - 1);
+            const uint32_t pos = s_base[d] + s_cnt[warp][d] + place[r];
+            if (!last) __stcg(kout + pos, key[r]);
+            __stcg(vout + pos, val[r]);
+        }
+        cur ^= 1;
+        // the entries are where the next pass reads them, and the totals are read
+        cluster.sync();
+    }
+    if (first) {   // equal keys throughout: the index order
+#pragma unroll
+        for (int r = 0; r < DC_ROUNDS; ++r)
+            if (r < R && e0 + 32 * r < NV) v0[e0 + 32 * r] = val[r];
+        cluster.sync();   // nobody leaves while its flags may still be read
+    }
+}
+
 // ------------------------------------------------------------- workspace
 struct BinWs {
     uint32_t *dk[2], *dv[2];
@@ -1103,6 +1274,13 @@ gs_status radix_sort_pairs(uint32_t *k[2], uint32_t *v[2], int64_t n, int bits, 
 static gs_status depth_sort(const float *depth, const int32_t *radius, int64_t NV, bool skip, const BinWs &w, int &cur,
                             cudaStream_t st)
 {
+    if (skip && NV <= DC_MAX_ENTRIES) {
+        cur = 0;
+        note_launch();
+        launch_next(depth_sort_cluster_kernel, DC_CTAS, DC_THREADS, 0, st, depth, radius, (int)NV, w.dk[0], w.dk[1],
+                    w.dv[0], w.dv[1], w.kor);
+        return launch_status("depth sort");
+    }
     const int G = (int)std::min<int64_t>(sort_blocks(), ceil_div(NV, SORT_TILE));
     cudaMemsetAsync(w.kor, 0, 2 * sizeof(uint32_t), st);
     note_launch();
