@@ -1013,19 +1013,21 @@ __global__ void __launch_bounds__(CS_THREADS) cs_place_kernel(CsParams p)
 // the warp's equal digits come from ballots and the warp's own row of
 // counters, the rows are scanned over the block's warps, and the blocks'
 // digit totals are read through distributed shared memory.  Entries pass
-// between the blocks through the sort's global buffers (L2).  The same
-// order, the same skipped bytes and the same buffers as the passes above.
-// What bounds it is the chain of a warp's rounds (about 1.4 us a round and
-// pass), so the limit is where the passes above catch up.  Whole binning, this
-// way against the launches, in a graph / in a stream: 1K entries 30 against 47 /
-// 30 against 48 us, 16K 38 / 51 and 39 / 68, 32K 49 / 53 and 50 / 71, 40K 55 /
-// 53 and 56 / 73, 64K 71 / 53 and 74 / 75.
-constexpr int DC_CTAS = 8, DC_THREADS = 1024, DC_WARPS = DC_THREADS / 32, DC_ROUNDS = 4;
+// between the blocks through the sort's global buffers (L2), (key, value) in
+// one 8-byte store: pairs_k is the two key buffers, pairs_v the two value
+// buffers, which follow one another in the workspace.  The same order, the
+// same skipped bytes and the values in the same buffer as the passes above.
+// What bounds it is the scattered stores (32 wavefronts an instruction, eight
+// SMs: about 1 us a round and pass), so the limit is where the passes above
+// catch up.  Whole binning, this way against the launches, in a graph / in a
+// stream: 1K entries 30 against 47 / 30 against 48 us, 16K 35 / 51 and 36 / 68,
+// 32K 43 / 53 and 44 / 71, 48K 51 / 53 and 56 / 73, 64K 59 / 53 and 63 / 75.
+constexpr int DC_CTAS = 8, DC_THREADS = 1024, DC_WARPS = DC_THREADS / 32, DC_ROUNDS = 6;
 constexpr int DC_ROW = RADIX + 1;   // a digit's counters of 8 w rows meet different banks
-constexpr int64_t DC_MAX_ENTRIES = (int64_t)DC_CTAS * DC_THREADS * DC_ROUNDS;   // 32 768
+constexpr int64_t DC_MAX_ENTRIES = (int64_t)DC_CTAS * DC_THREADS * DC_ROUNDS;   // 49 152
 
 __global__ void __cluster_dims__(DC_CTAS, 1, 1) __launch_bounds__(DC_THREADS)
-    depth_sort_cluster_kernel(const float *depth, const int32_t *radius, int NV, uint32_t *k0, uint32_t *k1,
+    depth_sort_cluster_kernel(const float *depth, const int32_t *radius, int NV, uint2 *pairs_k, uint2 *pairs_v,
                               uint32_t *v0, uint32_t *v1, uint32_t *kor)
 {
     if (grid_wait()) return;
@@ -1072,22 +1074,26 @@ __global__ void __cluster_dims__(DC_CTAS, 1, 1) __launch_bounds__(DC_THREADS)
         kor[0] = o1;
         kor[1] = o0;
     }
-    bool first = true;
-    int cur = 0;
+    int passes = 0;
+    for (int shift = 0; shift < 32; shift += 8) passes += ((diff >> shift) & (RADIX - 1)) != 0u;
+    // pass f of these writes pairs_k and pairs_v in turn, so that the last
+    // reads pairs_k, and the last the values into v0 or v1
+    int f = 0;
     for (int shift = 0; shift < 32; shift += 8) {
         if (((diff >> shift) & (RADIX - 1)) == 0u) continue;
-        if (!first) {
-            const uint32_t *kin = cur ? k1 : k0, *vin = cur ? v1 : v0;
+        uint2 *in = (passes - f) & 1 ? pairs_k : pairs_v, *out = (passes - f) & 1 ? pairs_v : pairs_k;
+        if (f > 0) {
 #pragma unroll
             for (int r = 0; r < DC_ROUNDS; ++r) {
                 const int e = e0 + 32 * r;
                 if (r < R && e < NV) {
-                    key[r] = __ldcg(kin + e);
-                    val[r] = __ldcg(vin + e);
+                    const uint2 x = __ldcg(in + e);
+                    key[r] = x.x;
+                    val[r] = x.y;
                 }
             }
         }
-        first = false;
+        ++f;
         uint32_t *cnt = s_cnt[warp];
         for (int d = lane; d < RADIX; d += 32) cnt[d] = 0u;
         __syncwarp();
@@ -1152,21 +1158,19 @@ __global__ void __cluster_dims__(DC_CTAS, 1, 1) __launch_bounds__(DC_THREADS)
             s_base[tid] = lower + before;
         }
         __syncthreads();
-        const bool last = (diff >> shift >> 8) == 0u;   // the placement after this reads the values only
-        uint32_t *kout = cur ? k0 : k1, *vout = cur ? v0 : v1;
+        uint32_t *vout = passes & 1 ? v1 : v0;
 #pragma unroll
         for (int r = 0; r < DC_ROUNDS; ++r) {
             if (r >= R || e0 + 32 * r >= NV) continue;
             const uint32_t d = (key[r] >> shift) & (RADIX - 1);
             const uint32_t pos = s_base[d] + s_cnt[warp][d] + place[r];
-            if (!last) __stcg(kout + pos, key[r]);
-            __stcg(vout + pos, val[r]);
+            if (f == passes) __stcg(vout + pos, val[r]);
+            else __stcg(out + pos, make_uint2(key[r], val[r]));
         }
-        cur ^= 1;
         // the entries are where the next pass reads them, and the totals are read
         cluster.sync();
     }
-    if (first) {   // equal keys throughout: the index order
+    if (passes == 0) {   // equal keys throughout: the index order
 #pragma unroll
         for (int r = 0; r < DC_ROUNDS; ++r)
             if (r < R && e0 + 32 * r < NV) v0[e0 + 32 * r] = val[r];
@@ -1277,8 +1281,8 @@ static gs_status depth_sort(const float *depth, const int32_t *radius, int64_t N
     if (skip && NV <= DC_MAX_ENTRIES) {
         cur = 0;
         note_launch();
-        launch_next(depth_sort_cluster_kernel, DC_CTAS, DC_THREADS, 0, st, depth, radius, (int)NV, w.dk[0], w.dk[1],
-                    w.dv[0], w.dv[1], w.kor);
+        launch_next(depth_sort_cluster_kernel, DC_CTAS, DC_THREADS, 0, st, depth, radius, (int)NV,
+                    reinterpret_cast<uint2 *>(w.dk[0]), reinterpret_cast<uint2 *>(w.dv[0]), w.dv[0], w.dv[1], w.kor);
         return launch_status("depth sort");
     }
     const int G = (int)std::min<int64_t>(sort_blocks(), ceil_div(NV, SORT_TILE));

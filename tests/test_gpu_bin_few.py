@@ -1,5 +1,5 @@
 """The binning's depth sort at and around the number of entries one cluster of
-blocks sorts (32 768): every view's list, with one bin a view, is its visible
+blocks sorts (49 152): every view's list, with one bin a view, is its visible
 entries in a stable sort of the depth bits, bit for bit."""
 import pytest
 import torch
@@ -14,8 +14,8 @@ W, H, BIN = 512, 480, 64
 
 @pytest.mark.parametrize("culled", [False, True])
 @pytest.mark.parametrize("depths", ["random", "one", "low byte", "high bytes"])
-@pytest.mark.parametrize("V,N", [(1, 1), (1, 33), (3, 700), (1, 8191), (2, 4097), (1, 24577), (5, 6553), (4, 8192),
-                                 (1, 32769)])
+@pytest.mark.parametrize("V,N", [(1, 1), (1, 33), (3, 700), (1, 8191), (2, 4097), (1, 40961), (5, 6553), (4, 12288),
+                                 (1, 49153)])
 def test_lists_are_stable_sorts_of_the_depth_bits(V, N, depths, culled):
     gen = torch.Generator(device=DEV).manual_seed(V * N)
     r = Rasterizer(N, V, W, H, V * N + 1, DEV, bin=BIN)
