@@ -96,8 +96,8 @@ __device__ __forceinline__ void walk_column(const float *const (&base)[N], int g
             float v[N];
 #pragma unroll
             for (int m = 0; m < N; ++m)
-                v[m] = __ldg(reinterpret_cast<const float *>(reinterpret_cast<const char *>(base[m]) +
-                                                             (i & 1 ? bottom : top)));
+                v[m] = *reinterpret_cast<const float *>(reinterpret_cast<const char *>(base[m]) +
+                                                        (i & 1 ? bottom : top));
             if (i & 1) bottom -= step;
             else top += step;
             f(inwards(i, ROWS), v);
@@ -111,7 +111,7 @@ __device__ __forceinline__ void walk_column(const float *const (&base)[N], int g
             const bool ok = okx && gy0 + k >= 0 && gy0 + k < H;
             float v[N];
 #pragma unroll
-            for (int m = 0; m < N; ++m) v[m] = ok ? __ldg(base[m] + at0 + (int64_t)k * W) : 0.f;
+            for (int m = 0; m < N; ++m) v[m] = ok ? base[m][at0 + (int64_t)k * W] : 0.f;
             f(k, v);
         }
     }
@@ -307,8 +307,8 @@ __global__ void __launch_bounds__(LTHREADS, 4) ssim_bwd_kernel(LossParams p)
     for (int i = 0; i < LR; ++i) {
         const bool ok = okx && y0 + tid / LC + i * RSTEP < p.H;
         const I at = first + (I)(i * RSTEP) * (I)p.W;
-        xv[i] = ok ? __ldg(X + at) : 0.f;
-        yv[i] = ok ? __ldg(Y + at) : 0.f;
+        xv[i] = ok ? X[at] : 0.f;
+        yv[i] = ok ? Y[at] : 0.f;
     }
     __syncthreads();
     if (!okx) return;

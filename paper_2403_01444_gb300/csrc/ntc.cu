@@ -344,11 +344,8 @@ __device__ __forceinline__ float adam_rate(const gs_adam &hp, int t)
 constexpr int ADAM_GROUPS = ADAM_GROUPS_N;
 
 template <int SHADOW>
-__global__ void ADAM_BOUNDS adam_kernel(float *__restrict__ p, float *__restrict__ g,
-                                                   float *__restrict__ m, float *__restrict__ v,
-                                                   int64_t n, gs_adam hp,
-                                                   const gs_train_state *__restrict__ st,
-                                                   void *__restrict__ shadow)
+__global__ void ADAM_BOUNDS adam_kernel(float *p, float *g, float *m, float *v, int64_t n, gs_adam hp,
+                                        const gs_train_state *st, void *shadow)
 {
     if (grid_wait()) return;
     const bool skip = st->found_inf != 0;

@@ -239,7 +239,7 @@ __device__ __forceinline__ void load_sh(const ProjectParams &p, int64_t i, float
         const float4 *s4 = reinterpret_cast<const float4 *>(shg);
 #pragma unroll
         for (int q = 0; q < N / 4; ++q) {
-            const float4 t = __ldg(s4 + q);
+            const float4 t = s4[q];
             sh[4 * q] = t.x;
             sh[4 * q + 1] = t.y;
             sh[4 * q + 2] = t.z;
@@ -247,7 +247,7 @@ __device__ __forceinline__ void load_sh(const ProjectParams &p, int64_t i, float
         }
     } else {
 #pragma unroll
-        for (int q = 0; q < N; ++q) sh[q] = __ldg(shg + q);
+        for (int q = 0; q < N; ++q) sh[q] = shg[q];
     }
 }
 
