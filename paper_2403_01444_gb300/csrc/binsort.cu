@@ -1355,17 +1355,17 @@ static gs_status count_sort_views(const gs_projected *proj, int64_t n, int v0, i
     cp.n_eff = w.n_eff;
     cp.vals = vals;
     cp.keys = keys;
-    const int smem_count = CS_WARPS * (cp.kp / 2) * (int)sizeof(uint32_t);
-    const int smem_place = cp.kp * (int)(sizeof(uint32_t) + CS_WARPS * sizeof(uint16_t));
-    set_smem_limit((const void *)cs_count_kernel, smem_count, st);
-    set_smem_limit((const void *)cs_place_kernel, smem_place, st);
+    auto smem_count = [](size_t kp) { return CS_WARPS * (kp / 2) * sizeof(uint32_t); };
+    auto smem_place = [](size_t kp) { return kp * (sizeof(uint32_t) + CS_WARPS * sizeof(uint16_t)); };
+    set_smem_limit((const void *)cs_count_kernel, smem_count(cs_pad_keys(CS_MAX_KEYS)));
+    set_smem_limit((const void *)cs_place_kernel, smem_place(cs_pad_keys(CS_MAX_KEYS)));
     note_launch();
-    launch_next(cs_count_kernel, G, CS_THREADS, smem_count, st, cp);
+    launch_next(cs_count_kernel, G, CS_THREADS, smem_count(cp.kp), st, cp);
     note_launch();
     const KeyBases kb{w.done, capacity, d_count, w.n_eff, d_err, ranges + 2 * (int64_t)v0 * bins, v0 > 0};
     launch_next(scan_digit_rows_kernel, nkeys, SORT_THREADS, 0, st, w.hist, G, nkeys, nullptr, 0, kb);
     note_launch();
-    launch_next(cs_place_kernel, G, CS_THREADS, smem_place, st, cp);
+    launch_next(cs_place_kernel, G, CS_THREADS, smem_place(cp.kp), st, cp);
     return launch_status("gs_bin_sort");
 }
 

@@ -56,11 +56,13 @@ inline bool stream_captures(cudaStream_t s)
     return cs != cudaStreamCaptureStatusNone;
 }
 
-// Raise a kernel's dynamic shared-memory limit, except while the stream is
-// being captured into a graph (the first, eager call has already done it).
-inline void set_smem_limit(const void *kernel, int bytes, cudaStream_t s)
+// A kernel's dynamic shared-memory limit.  It replaces the limit set before,
+// for every stream and thread, so each kernel is always given the same bytes:
+// the most that any of its launches takes.  It is no stream operation and may
+// be called during a capture.
+inline void set_smem_limit(const void *kernel, size_t bytes)
 {
-    if (!stream_captures(s)) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // Programmatic dependent launch: a kernel launched by launch_next may be set

@@ -115,8 +115,7 @@ __device__ __forceinline__ float4 mf_relu(const float2 (&a)[2])
 }
 
 // The activations of all layers share one buffer: with the weights it stays
-// below the 48 KB that a kernel has without asking (so that a first call may
-// be a captured one), and four blocks fit an SM.
+// below the 48 KB that a kernel has without asking, and four blocks fit an SM.
 template <typename ET>
 __global__ void __launch_bounds__(MF_THREADS, 4) mlp_f32_fwd_kernel(const ET *enc, bool vec, int64_t n,
                                                                     const float *W, float *raw7)
@@ -354,7 +353,7 @@ template <typename ET>
 static void launch_bwd(const void *enc, int64_t n, const gs_mlp *w, const float *d_raw7, const float *d_scale,
                        float *dW, float *d_enc, const uint32_t *rows, const int64_t *d_rows, cudaStream_t s)
 {
-    set_smem_limit((const void *)mlp_f32_bwd_kernel<ET>, (int)MF_BWD_SMEM, s);
+    set_smem_limit((const void *)mlp_f32_bwd_kernel<ET>, MF_BWD_SMEM);
     const int blocks = (int)std::min<int64_t>(ceil_div(n, MF_ROWS), 2 * num_sms());
     note_launch();
     mlp_f32_bwd_kernel<ET><<<blocks, MF_THREADS, MF_BWD_SMEM, s>>>((const ET *)enc, aligned(enc, 4 * sizeof(ET)), n,

@@ -679,7 +679,7 @@ static gs_status launch_fwd(TcParams p, cudaStream_t s)
     p.wait_tries = s_wait_tries.load();
     const size_t smem = sizeof(FwdSmem) + 1024;
     const int grid = (int)std::min<int64_t>(ceil_div(p.n, TM), num_sms() * 4);
-    set_smem_limit((const void *)mlp_tc_fwd_kernel<ET, FUSED>, (int)smem, s);
+    set_smem_limit((const void *)mlp_tc_fwd_kernel<ET, FUSED>, smem);
     note_launch();
     mlp_tc_fwd_kernel<ET, FUSED><<<grid, TM, smem, s>>>(p);
     return launch_status(FUSED ? "ntc_fused_fwd" : "ntc_mlp_fwd (tcgen05)");
@@ -691,7 +691,7 @@ static gs_status launch_bwd(TcParams p, cudaStream_t s)
     p.wait_tries = s_wait_tries.load();
     const size_t smem = sizeof(BwdSmem) + 1024;
     const int grid = (int)std::min<int64_t>(ceil_div(p.n, TM), num_sms() * 2);
-    set_smem_limit((const void *)mlp_tc_bwd_kernel<ET, FUSED>, (int)smem, s);
+    set_smem_limit((const void *)mlp_tc_bwd_kernel<ET, FUSED>, smem);
     note_launch();
     mlp_tc_bwd_kernel<ET, FUSED><<<grid, TM, smem, s>>>(p);
     return launch_status(FUSED ? "ntc_fused_bwd" : "ntc_mlp_bwd (tcgen05)");
