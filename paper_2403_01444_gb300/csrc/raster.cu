@@ -69,12 +69,17 @@ __device__ __forceinline__ float pair_gauss(float power)
     return g;
 }
 
-// alpha >= 1/255 (Eq. 4's skip) is tested on the base-2 power, power >=
-// -log2(255 o) staged with the record: forward and reverse take the same
-// decision, which differs from the test on alpha only within the rounding of
-// the exponential
 constexpr float kAlphaCap = 0.99f;
 constexpr float kTEps = 1e-4f;
+
+// alpha >= 1/255 (Eq. 4's skip) is tested on the base-2 power, -power <=
+// log2(255 o) staged with the record: forward and reverse take the same
+// decision, which differs from the test on alpha only within the rounding of
+// the exponential.  Only records with 255 o >= 1 are staged.  A logarithm
+// that rounds below 0, or to -0, at 255 o = 1 counts as +0, so that the
+// threshold's bit pattern is below those of every negative number and NaN.
+__device__ __forceinline__ bool visible(float o) { return o * 255.f >= 1.f; }
+__device__ __forceinline__ float staged_threshold(float o) { return fmaxf(__log2f(255.f * o), 0.f); }
 
 // Can record (m, co) reach alpha >= 1/255 at some pixel centre of tile
 // (tx_t, ty_t)?  alpha = o exp(-q/2) with q = A dx^2 + 2B dx dy + C dy^2, so
@@ -86,7 +91,7 @@ constexpr float kTEps = 1e-4f;
 // so images, gradients and list positions are unchanged.
 __device__ __forceinline__ bool ellipse_hits_tile(float2 m, float4 co, int tx_t, int ty_t)
 {
-    if (!(co.w * 255.f >= 1.f)) return false;
+    if (!visible(co.w)) return false;
     const float tau = 2.f * __logf(255.f * co.w) + 0.01f;
     const float xa = (float)(tx_t * 16) + 0.5f - m.x, xb = xa + 15.f;
     const float ya = (float)(ty_t * 16) + 0.5f - m.y, yb = ya + 15.f;
@@ -290,9 +295,7 @@ __global__ void __launch_bounds__(NT, 9) raster_fwd_kernel(RasterParams p)
             if (p.tl_rec && staged + slot < p.tl_cap)
                 p.tl_rec[tg * p.tl_cap + staged + slot] = make_uint2(g, (uint32_t)k);
             FwdBatch &B = s_batch[buf];
-            // a threshold below 0 (the logarithm's rounding at 255 o = 1) is one no pixel passes
-            const float thr = __log2f(255.f * co.w);
-            B.xyt[slot] = make_float4(thr >= 0.f ? m.x : nan, m.y, thr, 0.f);
+            B.xyt[slot] = make_float4(m.x, m.y, staged_threshold(co.w), 0.f);
             B.co[slot] = scale_conic(co);
             float *c = &B.rgbk[slot].x;
             const float *src = p.rgb + 3 * (vb + g);
@@ -727,10 +730,11 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
                 if (AHEAD) colour();
                 const float2 m = p.mean2d[vb + e.x];
                 co = p.conic_op[vb + e.x];
-                xyt = make_float4(m.x, m.y, __log2f(255.f * co.w), __uint_as_float(e.y));
+                xyt = make_float4(m.x, m.y, staged_threshold(co.w), __uint_as_float(e.y));
+                keep = visible(co.w);
                 co = scale_conic(co);
                 co.w = -co.w;
-                keep = xyt.z >= 0.f && staged_hits<NP>(xyt, co, cx0, cy0);
+                keep = keep && staged_hits<NP>(xyt, co, cx0, cy0);
             }
             const unsigned kept = __ballot_sync(all, keep);
             if (keep) {
