@@ -10,7 +10,7 @@
 // FMA pipes and not shared memory are the bound.  (One thread per row, with
 // the whole row's activations in its registers or its own shared-memory
 // column, reads a weight or an activation per multiply-add: 44 us forward and
-// 237 us reverse at 50 000 rows, against 25 and 67 us.  At 80 TFLOP/s they
+// 237 us reverse at 50 000 rows, against 25 and 65 us.  At 80 TFLOP/s they
 // would take 8 and 24 us: the barriers between a chunk's products and the last,
 // partly filled round of 782 chunks over the resident blocks are the rest.)
 //
@@ -114,6 +114,36 @@ __device__ __forceinline__ float4 mf_relu(const float2 (&a)[2])
     return make_float4(fmaxf(a[0].x, 0.f), fmaxf(a[0].y, 0.f), fmaxf(a[1].x, 0.f), fmaxf(a[1].y, 0.f));
 }
 
+// w[i][j] += sum over the chunk's rows of A[tr + 16 i][row] B[tc + 16 j][row]
+template <int NB>
+__device__ __forceinline__ void mf_contract(float (&w)[4][NB], const float *A, const float *B, int tr, int tc)
+{
+    float2 s[4][NB];   // over the even and the odd rows
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < NB; ++j) s[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int r = 0; r < MF_ROWS; r += 4) {
+        float4 a[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = mf_ld4(A + (tr + 16 * i) * MF_LD + r);
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            const float4 b = mf_ld4(B + (tc + 16 * j) * MF_LD + r);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                s[i][j] = __ffma2_rn(make_float2(a[i].x, a[i].y), make_float2(b.x, b.y), s[i][j]);
+                s[i][j] = __ffma2_rn(make_float2(a[i].z, a[i].w), make_float2(b.z, b.w), s[i][j]);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < NB; ++j) w[i][j] += s[i][j].x + s[i][j].y;
+}
+
 // The activations of all layers share one buffer: with the weights it stays
 // below the 48 KB that a kernel has without asking, and four blocks fit an SM.
 template <typename ET>
@@ -163,8 +193,11 @@ __global__ void __launch_bounds__(MF_THREADS, 4) mlp_f32_fwd_kernel(const ET *en
 }
 
 // One block runs the forward pass of a chunk again, then the row gradients
-// and, from registers that live over all its chunks, the weight gradients;
-// one atomic per weight (eight for the last layer's) and block at the end.
+// and the weight gradients.  These are summed in three levels, so that no chain
+// of additions grows with the rows of all chunks: a chunk's rows (the even and
+// the odd ones, 32 each; 8 a warp for the last layer), the chunks in registers
+// that live over all of them, and the blocks by one atomic a weight and block
+// at the end (the last layer's warps are added up before).
 template <typename ET>
 __global__ void __launch_bounds__(MF_THREADS, 2)
     mlp_f32_bwd_kernel(const ET *enc, bool vec, int64_t n, const float *W, const float *d_raw7, const float *d_scale,
@@ -177,15 +210,13 @@ __global__ void __launch_bounds__(MF_THREADS, 2)
     const float scale = d_scale ? *d_scale : 1.f;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int tr = (warp >> 1) * 4 + (lane >> 3), tc = (warp & 1) * 8 + (lane & 7);
-    float2 dw1[4][2], dw2[4][4];  // sums over the even and the odd rows
-    float dw3[4][4];
+    float dw1[4][2], dw2[4][4], dw3[4][4];   // sums over the chunks so far
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (j < 2) dw1[i][j] = make_float2(0.f, 0.f);
-            dw2[i][j] = make_float2(0.f, 0.f);
-            dw3[i][j] = 0.f;
+            if (j < 2) dw1[i][j] = 0.f;
+            dw2[i][j] = dw3[i][j] = 0.f;
         }
     const int64_t nslots = d_rows ? *d_rows : n;
     const int64_t nchunks = (nslots + MF_ROWS - 1) / MF_ROWS;
@@ -273,70 +304,61 @@ __global__ void __launch_bounds__(MF_THREADS, 2)
             }
         }
         // dW1[j][m] and dW2[j][k]: j = tr + 16 i, m and k = tc + 16 i
-#pragma unroll 1
-        for (int r = 0; r < MF_ROWS; r += 4) {
-            float4 a[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = mf_ld4(sG1 + (tr + 16 * i) * MF_LD + r);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const float4 b = mf_ld4(sX + (tc + 16 * j) * MF_LD + r);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    dw1[i][j] = __ffma2_rn(make_float2(a[i].x, a[i].y), make_float2(b.x, b.y), dw1[i][j]);
-                    dw1[i][j] = __ffma2_rn(make_float2(a[i].z, a[i].w), make_float2(b.z, b.w), dw1[i][j]);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = mf_ld4(sG2 + (tr + 16 * i) * MF_LD + r);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float4 b = mf_ld4(sH1 + (tc + 16 * j) * MF_LD + r);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    dw2[i][j] = __ffma2_rn(make_float2(a[i].x, a[i].y), make_float2(b.x, b.y), dw2[i][j]);
-                    dw2[i][j] = __ffma2_rn(make_float2(a[i].z, a[i].w), make_float2(b.z, b.w), dw2[i][j]);
-                }
-            }
-        }
+        mf_contract<2>(dw1, sG1, sX, tr, tc);
+        mf_contract<4>(dw2, sG2, sH1, tr, tc);
         // dW3[q][j]: each warp takes 8 of the rows, q = 4 (lane / 16) + i, j = lane % 16 + 16 i
+        {
+            float d[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) d[i][j] = 0.f;
 #pragma unroll 1
-        for (int r = 8 * warp; r < 8 * warp + 8; r += 4) {
-            float4 a[4];
+            for (int r = 8 * warp; r < 8 * warp + 8; r += 4) {
+                float4 a[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = mf_ld4(sGO + (4 * (lane >> 4) + i) * MF_LD + r);
+                for (int i = 0; i < 4; ++i) a[i] = mf_ld4(sGO + (4 * (lane >> 4) + i) * MF_LD + r);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float4 b = mf_ld4(sH2 + ((lane & 15) + 16 * j) * MF_LD + r);
+                for (int j = 0; j < 4; ++j) {
+                    const float4 b = mf_ld4(sH2 + ((lane & 15) + 16 * j) * MF_LD + r);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    dw3[i][j] = fmaf(a[i].x, b.x, dw3[i][j]);
-                    dw3[i][j] = fmaf(a[i].y, b.y, dw3[i][j]);
-                    dw3[i][j] = fmaf(a[i].z, b.z, dw3[i][j]);
-                    dw3[i][j] = fmaf(a[i].w, b.w, dw3[i][j]);
+                    for (int i = 0; i < 4; ++i) {
+                        d[i][j] = fmaf(a[i].x, b.x, d[i][j]);
+                        d[i][j] = fmaf(a[i].y, b.y, d[i][j]);
+                        d[i][j] = fmaf(a[i].z, b.z, d[i][j]);
+                        d[i][j] = fmaf(a[i].w, b.w, d[i][j]);
+                    }
                 }
             }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) dw3[i][j] += d[i][j];
         }
         __syncthreads();
+    }
+    float *sW3 = sX;   // the warps' sums of the last layer, [warp][8][64]; every chunk is done with sX to sH2
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            sW3[(warp * 8 + 4 * (lane >> 4) + i) * 64 + (lane & 15) + 16 * j] = dw3[i][j];
+    __syncthreads();
+    for (int k = t; k < 7 * 64; k += MF_THREADS) {
+        float s = 0.f;
+#pragma unroll
+        for (int w8 = 0; w8 < MF_THREADS / 32; ++w8) s += sW3[w8 * 8 * 64 + k];
+        if (s != 0.f) atomicAdd(dW + 64 * 32 + 64 * 64 + k, s);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int j = tr + 16 * i;
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const float s = dw1[i][k].x + dw1[i][k].y;
-            if (s != 0.f) atomicAdd(dW + j * 32 + tc + 16 * k, s);
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float s = dw2[i][k].x + dw2[i][k].y;
-            if (s != 0.f) atomicAdd(dW + 64 * 32 + j * 64 + tc + 16 * k, s);
-        }
-        const int q = 4 * (lane >> 4) + i;
+        for (int k = 0; k < 2; ++k)
+            if (dw1[i][k] != 0.f) atomicAdd(dW + j * 32 + tc + 16 * k, dw1[i][k]);
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-            if (q < 7 && dw3[i][k] != 0.f)
-                atomicAdd(dW + 64 * 32 + 64 * 64 + q * 64 + (lane & 15) + 16 * k, dw3[i][k]);
+            if (dw2[i][k] != 0.f) atomicAdd(dW + 64 * 32 + j * 64 + tc + 16 * k, dw2[i][k]);
     }
 }
 
