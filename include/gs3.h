@@ -201,7 +201,9 @@ GS_API gs_status gs_project(const gs_gaussians *g, const gs_camera *d_cams, int 
  * the transformed mean and rotation receive gradients).  grads[V][N][8] holds
  * dL/d(u, v, A, B, C, r, g, b) per (view, Gaussian) as written by
  * gs_raster_bwd.  Overwrites d_mean[N][3] and d_quat[N][4] (gradient wrt the
- * un-normalised input quaternion), summed over the V views. */
+ * un-normalised input quaternion), summed over the V views.  A Gaussian none of
+ * whose records has a gradient gets zeros for V <= 32, whatever its SH
+ * coefficients, unless its rotation or its covariance is not finite. */
 GS_API gs_status gs_project_bwd(const gs_gaussians *g, const gs_camera *d_cams, int V, int W, int H,
                          const float *grads, float *d_mean, float *d_quat, gs_stream stream);
 

@@ -615,11 +615,12 @@ __global__ void __launch_bounds__(PB_GAUSS) project_bwd_seen_kernel(ProjectParam
                       b.z == 0.f && b.w == 0.f);
         }
         // a rotation or scales that make no finite covariance go through the
-        // arithmetic, which says so in the gradient
+        // arithmetic, which says so in the gradient (1e38: the squares of the
+        // scales, with room for the rounding of the rotation's entries)
         const float4 q = reinterpret_cast<const float4 *>(p.quat)[i];
         const float iq = 1.f / sqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
-        seen |= !(iq > 0.f && isfinite(iq) && isfinite(p.scale[3 * i]) && isfinite(p.scale[3 * i + 1]) &&
-                  isfinite(p.scale[3 * i + 2]));
+        const float s0 = p.scale[3 * i], s1 = p.scale[3 * i + 1], s2 = p.scale[3 * i + 2];
+        seen |= !(iq > 0.f && isfinite(iq) && s0 * s0 + s1 * s1 + s2 * s2 <= 1e38f);
         if (!seen) {
             p.d_mean[3 * i] = p.d_mean[3 * i + 1] = p.d_mean[3 * i + 2] = 0.f;
             reinterpret_cast<float4 *>(p.d_quat)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
