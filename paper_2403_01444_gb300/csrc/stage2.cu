@@ -141,10 +141,11 @@ __global__ void __cluster_dims__(SEL_CTAS, 1, 1) __launch_bounds__(SEL_THREADS)
 #pragma unroll
             for (int u = 0; u < SEL_U; ++u) {
                 // the division only where the product does not rule it out (by more
-                // than the roundings of both): a division for every value of both
-                // walks took half of the time
+                // than the roundings of both; an infinite product, whose bound is
+                // no number, rules nothing out): a division for every value of
+                // both walks took half of the time
                 const float t = tau * (float)d[u];
-                bool in = d[u] > 0 && a[u] >= t - fabsf(t) * 1e-5f;
+                bool in = d[u] > 0 && !(a[u] < t - fabsf(t) * 1e-5f);
                 if (in) in = a[u] / (float)d[u] > tau;
                 f(j0 + 32 * u, __ballot_sync(0xffffffffu, in));
             }
