@@ -311,7 +311,8 @@ GS_API gs_status gs_raster_fwd(const gs_projected *proj, int64_t n, int V, int W
  * warp's pixels (a half or a quarter of a tile) before the FP32 atomics.
  * Overwrites grads[V][N][8] = dL/d(u, v, A, B, C, r, g, b) and, when non-NULL,
  * d_opacity[V][N].  bg is a host array of 3 floats.  d_stats (device
- * uint64[2], or NULL) accumulates the pairs walked and the pairs that had
+ * uint64[2], or NULL) accumulates the pairs walked (of each pixel, the records
+ * of its tile's list before its last contributor) and the pairs that had
  * contributed.  lists (or NULL): written by the gs_raster_fwd call on the same
  * proj, n, V, W, H, bin, vals and ranges; the reverse then stages a tile's
  * records from its list instead of testing its bin's list again (a tile with

@@ -467,8 +467,7 @@ __device__ __forceinline__ float2 weigh(float2 w, float2 d, float2 a)
 // -dL/dpower and of minus the weight.
 template <int NP, bool WANT_OP, bool STATS, bool GUARD>
 __device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, PixBwd<NP> &P, int head, int cnt, float pxf,
-                                          const float2 (&pyf)[NP], float cx0, int64_t vb, uint32_t &n_tested,
-                                          uint32_t &n_contrib)
+                                          const float2 (&pyf)[NP], float cx0, int64_t vb, uint32_t &n_contrib)
 {
     constexpr unsigned all = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -490,10 +489,7 @@ __device__ __forceinline__ void bwd_chunk(const RasterParams &p, BwdWarp &S, Pix
             const float2 np = __ffma2_rn(f2(0.5f), q, __fmul2_rn(f2(co.y), __fmul2_rn(f2(dx), dy[h])));
             const bool in0 = pos < P.last[2 * h] && __float_as_uint(np.x) <= thr;
             const bool in1 = pos < P.last[2 * h + 1] && __float_as_uint(np.y) <= thr;
-            if (STATS) {
-                n_tested += (pos < P.last[2 * h]) + (pos < P.last[2 * h + 1]);
-                n_contrib += (uint32_t)in0 + (uint32_t)in1;
-            }
+            if (STATS) n_contrib += (uint32_t)in0 + (uint32_t)in1;
             // minus alpha, before and after the cap
             float2 raw = __fmul2_rn(f2(co.w), make_float2(pair_gauss(-np.x), pair_gauss(-np.y)));
             raw.x = in0 ? raw.x : 0.f;
@@ -720,6 +716,7 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
                 cands -= take;
             }
             bool keep = (int)e.y < wlast;
+            int walked = 0x7fffffff;   // STATS: the position of a record of the tile's list
             float4 xyt, co;
             float c0 = 0.f, c1 = 0.f, c2 = 0.f;
             auto colour = [&]() {
@@ -730,11 +727,19 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
                 if (AHEAD) colour();
                 const float2 m = p.mean2d[vb + e.x];
                 co = p.conic_op[vb + e.x];
+                if (STATS && (listed >= 0 || ellipse_hits_tile(m, co, tx_t, ty_t))) walked = (int)e.y;
                 xyt = make_float4(m.x, m.y, staged_threshold(co.w), __uint_as_float(e.y));
                 keep = visible(co.w);
                 co = scale_conic(co);
                 co.w = -co.w;
                 keep = keep && staged_hits<NP>(xyt, co, cx0, cy0);
+            }
+            if (STATS) {
+                for (int l = 0; l < 32; ++l) {
+                    const int pos = __shfl_sync(all, walked, l);
+#pragma unroll
+                    for (int k = 0; k < 2 * NP; ++k) n_tested += pos < P.last[k];
+                }
             }
             const unsigned kept = __ballot_sync(all, keep);
             if (keep) {
@@ -755,9 +760,9 @@ __global__ void __launch_bounds__(32 * BWD_WARPS) raster_bwd_kernel(RasterParams
         }
         __syncwarp();
         if (guard)
-            bwd_chunk<NP, WANT_OP, STATS, true>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_tested, n_contrib);
+            bwd_chunk<NP, WANT_OP, STATS, true>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_contrib);
         else
-            bwd_chunk<NP, WANT_OP, STATS, false>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_tested, n_contrib);
+            bwd_chunk<NP, WANT_OP, STATS, false>(p, S, P, head, cnt, pxf, pyf, cx0, vb, n_contrib);
         head += BWD_CHUNK;
         if (head == BWD_QUEUE) head = 0;
         have -= cnt;
