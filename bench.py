@@ -12,6 +12,10 @@ available) resident in HBM; the per-iteration working set (pair buffers of
 ~0.5 GB) exceeds the 129 MB L2, so no flush is needed between iterations.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
+
+Standard output holds one line of JSON, the headline; the whole record, with
+the curves and the per-frame rows, goes to standard error before it as one
+line that starts with "record ".
 """
 from __future__ import annotations
 
@@ -736,10 +740,26 @@ def run_ours(args):
                 "e2e": {"value": e2e_ms * ITERS_PER_FRAME / 1e3, "unit": "s/frame",
                         "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": 4},
                 "gpu_launches": int(launches), "tc_timeouts": gs3.gs_tc_timeouts(), "clocks": clocks}
-        print(json.dumps(line), flush=True)
+        print("record " + json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if world > 1:
         torch.distributed.barrier()
         torch.distributed.destroy_process_group()
+
+
+def headline(record):
+    """The line of standard output: the record without its lists and with one
+    number a side workload, short enough for a reader that keeps a few KB."""
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "train_it_per_s", "full_frame_s", "raster_fwd_bwd_it_per_s",
+            "speedup_vs_plain_per_iter", "stages_ms", "roofline", "e2e", "gpu_launches", "tc_timeouts", "clocks")
+    line = {k: record[k] for k in keys}
+    for name, key in (("equal_psnr", "speedup_at_equal_psnr"), ("render_only", "fps"), ("stage2", "ms_per_iter"),
+                      ("stream", "s_per_frame"), ("large", "ms_per_iter")):
+        line[name] = {key: record[name][key]} if record[name] else None
+    cpu = record["cpu_baseline"]
+    line["cpu_baseline"] = cpu and {k: v for k, v in cpu.items() if k != "other_workloads"}
+    return line
 
 
 def stage2_workload(dev, warm_iters=300):
