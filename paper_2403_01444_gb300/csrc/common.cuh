@@ -79,9 +79,9 @@ inline void set_smem_limit(const void *kernel, size_t bytes)
 // 172 us, 338 -> 347 us), so a capturing stream gets ordinary launches.
 // The result is always 0: used as `if (grid_wait()) return;` it puts the loads
 // of inputs into a block of their own, above which the compiler cannot lift
-// them.  They are plain loads: __ldg and __restrict__ allow the read-only load,
-// which asks that its data not change while the kernel runs, and the kernel
-// before still writes them when this one starts.
+// them.  They are plain loads: __ldg, and __restrict__ on data that is only
+// read, allow the read-only load, which asks that its data not change while the
+// kernel runs, and the kernel before still writes them when this one starts.
 __device__ __forceinline__ unsigned grid_wait()
 {
     unsigned never;
