@@ -587,32 +587,59 @@ __global__ void __launch_bounds__(128) project_bwd_views_kernel(ProjectParams p)
 // Every Gaussian's mean and rotation (Stage 1).  Most records have no gradient
 // at all (hidden, or on no pixel: 85 to 95 % of the Gaussians in every view of
 // a batch), and a Gaussian without one has the gradient zero.  A block looks
-// through the record gradients of 128 Gaussians, a thread each, writes those
-// zeros and puts the others into a list, which its groups of lanes then work
-// through: the projection, whose arithmetic bounds the kernel, is formed again
-// only where it is needed, and the SH coefficients are read only there.
+// through the record gradients of its Gaussians, writes those zeros and puts the
+// others into a list, which its groups of lanes then work through: the
+// projection, whose arithmetic bounds the kernel, is formed again only where it
+// is needed, and the SH coefficients are read only there.
 // 250K Gaussians of degree 3, four 1352x1014 views 54 -> 25 us a training step;
 // 1M, sixteen 1920x1080 views 814 -> 202 us.
-constexpr int PB_GAUSS = 128;
+// A block takes G = 2^gbits Gaussians.  Where all of them have a gradient in
+// every view it works through G VP / 128 rounds, and 128 Gaussians a block are
+// too few blocks for a small set seen by many views: 3K Gaussians, 32 views, all
+// with a gradient, degree 3: 57 us, with 4 a block 9 us.  So G is halved down to
+// one round while there are fewer than 4 blocks an SM, and down to eight rounds
+// while there are fewer than 8 (250K and more keep 128, where most Gaussians
+// have none).  All with a gradient / a tenth of them, degree 0, 128 a block ->
+// this rule, beside a launch of one round a block that projects all: 50K in 16
+// views 45 -> 32 / 11 -> 10 us, beside 26 / 26; 50K in 32 views 96 -> 52 / 21 -> 14,
+// beside 48 / 48; 25K in 8 views 19 -> 11 / 7.7 -> 7.6, beside 14 / 14.
+constexpr int PB_THREADS = 128;
+
+static int seen_gbits(int64_t n, int VP)
+{
+    int b = 7;
+    for (; (VP << b) > PB_THREADS; --b) {
+        const int64_t blocks = ceil_div(n, int64_t(1) << b);
+        if (blocks >= ((VP << b) > 8 * PB_THREADS ? 8 : 4) * (int64_t)num_sms()) break;
+    }
+    return b;
+}
 
 template <int DEG, int VP>
-__global__ void __launch_bounds__(PB_GAUSS) project_bwd_seen_kernel(ProjectParams p)
+__global__ void __launch_bounds__(PB_THREADS) project_bwd_seen_kernel(ProjectParams p, int gbits)
 {
     if (grid_wait()) return;
     extern __shared__ gs_camera s_cams[];
-    __shared__ uint8_t s_list[PB_GAUSS];
-    __shared__ int s_cnt[PB_GAUSS / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = threadIdx.x; k < p.V; k += blockDim.x) s_cams[k] = p.cams[k];
-    const int64_t j0 = (int64_t)blockIdx.x * PB_GAUSS, i = j0 + threadIdx.x;
+    __shared__ uint8_t s_any[PB_THREADS], s_list[PB_THREADS];
+    __shared__ int s_cnt[PB_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int k = tid; k < p.V; k += PB_THREADS) s_cams[k] = p.cams[k];
+    // thread = (Gaussian, every step-th view)
+    const int G = 1 << gbits, step = PB_THREADS >> gbits, j = tid & (G - 1);
+    const int64_t j0 = (int64_t)blockIdx.x * G, i = j0 + j;
     bool seen = false;
     if (i < p.n) {
         const float4 *gp = reinterpret_cast<const float4 *>(p.grads) + 2 * i;
-#pragma unroll 4
-        for (int v = 0; v < p.V; ++v) {
+        auto look = [&](int v) {
             const float4 a = gp[2 * (int64_t)v * p.n], b = gp[2 * (int64_t)v * p.n + 1];
             seen |= !(a.x == 0.f && a.y == 0.f && a.z == 0.f && a.w == 0.f && b.x == 0.f && b.y == 0.f &&
                       b.z == 0.f && b.w == 0.f);
+        };
+        if (step == 1) {
+#pragma unroll 4
+            for (int v = 0; v < p.V; ++v) look(v);
+        } else {
+            for (int v = tid >> gbits; v < p.V; v += step) look(v);
         }
         // a rotation or scales that make no finite covariance go through the
         // arithmetic, which says so in the gradient (1e38: the squares of the
@@ -621,25 +648,32 @@ __global__ void __launch_bounds__(PB_GAUSS) project_bwd_seen_kernel(ProjectParam
         const float iq = 1.f / sqrtf(q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w);
         const float s0 = p.scale[3 * i], s1 = p.scale[3 * i + 1], s2 = p.scale[3 * i + 2];
         seen |= !(iq > 0.f && isfinite(iq) && s0 * s0 + s1 * s1 + s2 * s2 <= 1e38f);
-        if (!seen) {
-            p.d_mean[3 * i] = p.d_mean[3 * i + 1] = p.d_mean[3 * i + 2] = 0.f;
-            reinterpret_cast<float4 *>(p.d_quat)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+    }
+    if (step > 1) {   // what the threads of a Gaussian found, to its first thread
+        s_any[tid] = 0;
+        __syncthreads();
+        if (seen) s_any[j] = 1;
+        __syncthreads();
+        seen = tid < G && s_any[tid];
+    }
+    if (tid < G && i < p.n && !seen) {
+        p.d_mean[3 * i] = p.d_mean[3 * i + 1] = p.d_mean[3 * i + 2] = 0.f;
+        reinterpret_cast<float4 *>(p.d_quat)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     const unsigned m = __ballot_sync(0xffffffffu, seen);
     if (lane == 0) s_cnt[warp] = __popc(m);
     __syncthreads();
     int off = 0, total = 0;
 #pragma unroll
-    for (int w = 0; w < PB_GAUSS / 32; ++w) {
+    for (int w = 0; w < PB_THREADS / 32; ++w) {
         off += w < warp ? s_cnt[w] : 0;
         total += s_cnt[w];
     }
-    if (seen) s_list[off + __popc(m & ((1u << lane) - 1u))] = (uint8_t)threadIdx.x;
+    if (seen) s_list[off + __popc(m & ((1u << lane) - 1u))] = (uint8_t)tid;
     __syncthreads();
-    const int v = threadIdx.x % VP;
+    const int v = tid % VP;
     // a warp's groups take consecutive entries
-    for (int k0 = warp * (32 / VP); k0 < total; k0 += PB_GAUSS / VP) {
+    for (int k0 = warp * (32 / VP); k0 < total; k0 += PB_THREADS / VP) {
         const int k = k0 + lane / VP;
         const bool live = k < total;
         const int64_t g = j0 + (live ? s_list[k] : 0);
@@ -655,8 +689,11 @@ static void launch_bwd_views(const ProjectParams &p, size_t shm, cudaStream_t s)
         constexpr int VP = decltype(vp)::value;
         if constexpr (FULL)
             launch_next(project_bwd_views_kernel<DEG, VP>, (unsigned)ceil_div(p.count * VP, threads), threads, shm, s, p);
-        else
-            launch_next(project_bwd_seen_kernel<DEG, VP>, (unsigned)ceil_div(p.n, PB_GAUSS), PB_GAUSS, shm, s, p);
+        else {
+            const int gbits = seen_gbits(p.n, VP);
+            launch_next(project_bwd_seen_kernel<DEG, VP>, (unsigned)ceil_div(p.n, int64_t(1) << gbits), PB_THREADS, shm,
+                        s, p, gbits);
+        }
     };
     if (p.V <= 1) go(std::integral_constant<int, 1>());
     else if (p.V <= 2) go(std::integral_constant<int, 2>());
