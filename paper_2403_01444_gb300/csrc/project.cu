@@ -443,7 +443,6 @@ __device__ __forceinline__ void bwd_finish(const ProjectParams &p, const GaussLo
 template <bool FULL, int DEG>
 __global__ void __launch_bounds__(128) project_bwd_kernel(ProjectParams p)
 {
-    if (grid_wait()) return;
     constexpr int K = (DEG + 1) * (DEG + 1);
     extern __shared__ gs_camera s_cams[];
     for (int k = threadIdx.x; k < p.V; k += blockDim.x) s_cams[k] = p.cams[k];
@@ -703,13 +702,25 @@ static void launch_bwd_views(const ProjectParams &p, size_t shm, cudaStream_t s)
     else go(std::integral_constant<int, 32>());
 }
 
-// More views than lanes: a thread per Gaussian walks them.
+// A thread per Gaussian walks the views where they are more than a warp's lanes,
+// and for the reverse of every parameter where the Gaussians alone fill the chip
+// and have few SH coefficients: then the lanes' sums over the views cost more
+// than walking does.  Thread / lanes, 250K Gaussians of degree 0: two views 17 /
+// 18 us, four 27 / 35, sixteen 110 / 188; degree 1: four 48 / 49, sixteen 164 /
+// 292.  Below the line, degree 0: eight views of 20K 15 / 9, four of 50K 13 / 10;
+// degree 1: four of 100K 27 / 20, eight of 50K 24 / 22.  Degree 2 and 3, whose
+// sums a thread keeps in global memory, are faster on lanes throughout (degree 2:
+// 250K in four views 156 / 83 us, in 32 953 / 885).
+// Its few, long blocks are launched in the ordinary way: set up before the grid
+// in front has ended they crowd the SMs that come free first (50K in 32 views, a
+// chain of such calls, 48 -> 62 us).
 template <bool FULL>
 static void launch_bwd(const ProjectParams &p, cudaStream_t s)
 {
     const int threads = 128;
     const size_t shm = sizeof(gs_camera) * p.V;
-    if (p.V <= 32) {
+    const bool thread_each = FULL && p.deg <= 1 && p.V > 1 && p.count >= 32768 && (p.count * p.V >> p.deg) >= 400000;
+    if (p.V <= 32 && !thread_each) {
         switch (p.deg) {
         case 0: launch_bwd_views<FULL, 0>(p, shm, s); break;
         case 1: launch_bwd_views<FULL, 1>(p, shm, s); break;
@@ -720,10 +731,10 @@ static void launch_bwd(const ProjectParams &p, cudaStream_t s)
     }
     const int blocks = (int)ceil_div(FULL ? p.count : p.n, threads);
     switch (p.deg) {
-    case 0: launch_next(project_bwd_kernel<FULL, 0>, blocks, threads, shm, s, p); break;
-    case 1: launch_next(project_bwd_kernel<FULL, 1>, blocks, threads, shm, s, p); break;
-    case 2: launch_next(project_bwd_kernel<FULL, 2>, blocks, threads, shm, s, p); break;
-    default: launch_next(project_bwd_kernel<FULL, 3>, blocks, threads, shm, s, p); break;
+    case 0: project_bwd_kernel<FULL, 0><<<blocks, threads, shm, s>>>(p); break;
+    case 1: project_bwd_kernel<FULL, 1><<<blocks, threads, shm, s>>>(p); break;
+    case 2: project_bwd_kernel<FULL, 2><<<blocks, threads, shm, s>>>(p); break;
+    default: project_bwd_kernel<FULL, 3><<<blocks, threads, shm, s>>>(p); break;
     }
 }
 

@@ -1,6 +1,11 @@
-"""The projection reverse on both sides of the lines at which a block takes more
-Gaussians.  It does a Gaussian's arithmetic the same way in every block size, so
-a call over all rows equals calls over a few of them bit for bit."""
+"""The projection reverses on both sides of the lines at which a block takes more
+Gaussians and at which a thread walks a Gaussian's views by itself.
+
+The reverse for mean and rotation does a Gaussian's arithmetic the same way in
+every block size, so a call over all rows equals calls over a few of them bit
+for bit.  The reverse of every parameter sums at most 32 views in another
+order: 1e-5 of a tensor's norm (33 roundings of 2^-24 of terms of either
+sign)."""
 import numpy as np
 import pytest
 import torch
@@ -44,3 +49,21 @@ def test_mean_and_rotation_do_not_depend_on_the_block(V, N, frac):
         gs3.gs_project_bwd(_rows(g, a, b), cams, V, W, H, grads[:, a:b].contiguous(), pm, pq)
         assert torch.equal(pm, dm[a:b]) and torch.equal(pq, dq[a:b])
 
+
+@pytest.mark.parametrize("deg,V,N", [(0, 2, 210_000), (0, 4, 101_000), (0, 16, 32_768), (0, 16, 32_767), (1, 4, 200_001),
+                                     (1, 32, 33_000), (2, 16, 60_000)])
+def test_every_parameter_whichever_kernel(deg, V, N):
+    g, cams, grads = _inputs(V, N, deg, 0.7)
+    op = torch.randn(V, N, device=DEV, generator=torch.Generator(device=DEV).manual_seed(1))
+    K = (deg + 1) ** 2
+
+    def run(first, count):
+        o = [torch.full(s, 7.0, device=DEV) for s in ((count, 3), (count, 4), (count, 3), (count,), (count, K, 3))]
+        gs3.gs_project_bwd_full(g, cams, V, W, H, grads, op, first, count, *o)
+        return o
+
+    whole = run(0, N)
+    for a, b in ((0, 1000), (N - 3001, N)):
+        for x, y in zip(whole, run(a, b - a)):
+            x, y = x[a:b].double(), y.double()
+            assert bool(torch.isfinite(x).all()) and float((x - y).norm()) <= 1e-5 * float(y.norm())
