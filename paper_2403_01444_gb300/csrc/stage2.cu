@@ -181,22 +181,28 @@ __global__ void __cluster_dims__(SEL_CTAS, 1, 1) __launch_bounds__(SEL_THREADS)
 
 // ------------------------------------------------------------------ spawn
 // The row kernels below (spawn, Adam, render) take a thread per column of a
-// row, ROW_T threads (>= 59 columns) a row and ROW_N rows a block, so that rows
-// and moments are read and written in whole lines and a few thousand rows
-// fill the chip.  With a thread per row each access touched a line per lane
-// and 3 000 rows were 24 blocks (Adam 91 us, now 4.9 us; spawn 35 us, now
-// 5.5 us; render 16 us, now 2 us).
-constexpr int ROW_T = 64, ROW_N = 4;
-static_assert(GS_ADDED_COLS(16) <= ROW_T, "a thread per column");
+// row, as many threads a row as the power of two that holds its columns (14 to
+// 59), so that rows and moments are read and written in whole lines and a few
+// thousand rows fill the chip.  With a thread per row each access touches a line
+// per lane and 3 000 rows are 24 blocks (degree 3: Adam 91 us, here 4.9 us;
+// spawn 35 us, here 5.5 us; render 16 us, here 2 us).
+constexpr int ROW_THREADS = 256;
 
-__global__ void __launch_bounds__(ROW_T *ROW_N) spawn_kernel(gs_gaussians src, const int32_t *idx,
-                                                             const int64_t *d_nsel, const float *z, float opl_init,
-                                                             gs_added dst, int64_t *d_nadd, int32_t *d_err)
+static dim3 row_block(int sh_deg)
+{
+    const int P = added_cols((sh_deg + 1) * (sh_deg + 1)), T = P <= 16 ? 16 : P <= 32 ? 32 : 64;
+    return dim3(T, ROW_THREADS / T);
+}
+static_assert(GS_ADDED_COLS(16) <= 64, "a thread per column");
+
+__global__ void __launch_bounds__(ROW_THREADS) spawn_kernel(gs_gaussians src, const int32_t *idx,
+                                                            const int64_t *d_nsel, const float *z, float opl_init,
+                                                            gs_added dst, int64_t *d_nadd, int32_t *d_err)
 {
     const int64_t nsel = *d_nsel, n0 = *d_nadd;
     const int K = (src.sh_deg + 1) * (src.sh_deg + 1), P = added_cols(K), q = threadIdx.x;
     if (q >= P) return;
-    for (int64_t k = (int64_t)blockIdx.x * ROW_N + threadIdx.y; k < nsel; k += (int64_t)gridDim.x * ROW_N) {
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; k < nsel; k += (int64_t)gridDim.x * blockDim.y) {
         const int64_t row = n0 + k;
         if (row >= dst.capacity) {
             if (q == 0) *d_err = GS_ERR_CAPACITY;
@@ -302,12 +308,12 @@ struct AdamLr {
     float lr[6];
 };
 
-__global__ void __launch_bounds__(ROW_T *ROW_N)
+__global__ void __launch_bounds__(ROW_THREADS)
     added_adam_kernel(gs_added a, int64_t n, const float *d_mean, const float *d_quat, const float *d_scale,
                       const float *d_ologit, const float *d_sh, AdamLr lr, float b1, float b2, float eps,
                       const gs_train_state *st, gs_gaussians out, int64_t out_first)
 {
-    const int64_t j = (int64_t)blockIdx.x * ROW_N + threadIdx.y;
+    const int64_t j = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
     const int K = (a.sh_deg + 1) * (a.sh_deg + 1), P = added_cols(K), q = threadIdx.x;
     if (j >= n || q >= P) return;
     const int64_t at = j * P + q;
@@ -344,13 +350,36 @@ __global__ void __launch_bounds__(ROW_T *ROW_N)
     column_to_render(x, q, K, out, out_first + j);
 }
 
-__global__ void __launch_bounds__(ROW_T *ROW_N) added_render_kernel(gs_added a, int64_t n, gs_gaussians out,
-                                                                    int64_t out_first)
+__global__ void __launch_bounds__(ROW_THREADS) added_render_kernel(gs_added a, int64_t n, gs_gaussians out,
+                                                                   int64_t out_first)
 {
-    const int64_t j = (int64_t)blockIdx.x * ROW_N + threadIdx.y;
+    const int64_t j = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
     const int K = (a.sh_deg + 1) * (a.sh_deg + 1), P = added_cols(K), q = threadIdx.x;
     if (j >= n || q >= P) return;
     column_to_render(a.rows[j * P + q], q, K, out, out_first + j);
+}
+
+// A thread per row, for very many rows of few columns: there a warp's columns go
+// to five arrays, a few lanes a store, and the stores are what it waits for
+// (500K rows of degree 0: a thread per column 25 us, per row 14; degree 1: 47, 40;
+// 100K of degree 1: 13, 11; at 20K of either 6, 10).
+constexpr int RENDER_ROWS = 128;
+
+__global__ void __launch_bounds__(RENDER_ROWS) added_render_rows_kernel(gs_added a, int64_t n, gs_gaussians out,
+                                                                        int64_t out_first)
+{
+    const int64_t j = (int64_t)blockIdx.x * RENDER_ROWS + threadIdx.x, o = out_first + j;
+    if (j >= n) return;
+    const int K = (a.sh_deg + 1) * (a.sh_deg + 1);
+    const float *r = a.rows + j * added_cols(K);
+    float *mean = const_cast<float *>(out.mean) + 3 * o, *scale = const_cast<float *>(out.scale) + 3 * o;
+    float *sh = const_cast<float *>(out.sh) + 3 * K * o;
+    for (int q = 0; q < 3; ++q) mean[q] = r[COL_MEAN + q];
+    reinterpret_cast<float4 *>(const_cast<float *>(out.quat))[o] =
+        make_float4(r[COL_QUAT], r[COL_QUAT + 1], r[COL_QUAT + 2], r[COL_QUAT + 3]);
+    for (int q = 0; q < 3; ++q) scale[q] = expf(r[COL_LOGS + q]);
+    const_cast<float *>(out.opacity_logit)[o] = r[COL_OPL];
+    for (int q = 0; q < 3 * K; ++q) sh[q] = r[COL_SH + q];
 }
 
 static bool added_ok(const gs_added *a)
@@ -401,7 +430,7 @@ extern "C" gs_status gs_added_spawn(const gs_gaussians *src, const int32_t *idx,
     cudaStream_t s = as_stream(stream);
     const float opl = logf(opacity_init / (1.f - opacity_init));
     note_launch();
-    spawn_kernel<<<num_sms() * 8, dim3(ROW_T, ROW_N), 0, s>>>(*src, idx, d_nsel, z, opl, *dst, d_nadd, d_err);
+    spawn_kernel<<<num_sms() * 8, row_block(dst->sh_deg), 0, s>>>(*src, idx, d_nsel, z, opl, *dst, d_nadd, d_err);
     note_launch();
     spawn_count_kernel<<<1, 1, 0, s>>>(d_nsel, dst->capacity, d_nadd);
     return launch_status("gs_added_spawn");
@@ -444,7 +473,8 @@ extern "C" gs_status gs_added_adam(gs_added *a, int64_t n, const float *d_mean, 
     AdamLr l;
     for (int k = 0; k < 6; ++k) l.lr[k] = lr[k];
     note_launch();
-    added_adam_kernel<<<(int)ceil_div(n, ROW_N), dim3(ROW_T, ROW_N), 0, as_stream(stream)>>>(
+    const dim3 block = row_block(a->sh_deg);
+    added_adam_kernel<<<(int)ceil_div(n, block.y), block, 0, as_stream(stream)>>>(
         *a, n, d_mean, d_quat, d_scale, d_opacity_logit, d_sh, l, beta1, beta2, eps, d_state, *out,
         out_first);
     return launch_status("gs_added_adam");
@@ -459,6 +489,11 @@ extern "C" gs_status gs_added_to_render(const gs_added *a, int64_t n, const gs_g
     GS_REQUIRE(out->sh_deg == a->sh_deg && aligned(out->quat, 16), "gs_added_to_render: bad output set");
     if (n == 0) return GS_OK;
     note_launch();
-    added_render_kernel<<<(int)ceil_div(n, ROW_N), dim3(ROW_T, ROW_N), 0, as_stream(stream)>>>(*a, n, *out, out_first);
+    const dim3 block = row_block(a->sh_deg);
+    cudaStream_t s = as_stream(stream);
+    if (a->sh_deg <= 1 && n >= 65536)
+        added_render_rows_kernel<<<(int)ceil_div(n, RENDER_ROWS), RENDER_ROWS, 0, s>>>(*a, n, *out, out_first);
+    else
+        added_render_kernel<<<(int)ceil_div(n, block.y), block, 0, s>>>(*a, n, *out, out_first);
     return launch_status("gs_added_to_render");
 }
