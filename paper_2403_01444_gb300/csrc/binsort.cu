@@ -712,7 +712,7 @@ constexpr int CS_MAX_ENTRIES = 4095;     // entries per warp at most: CS_WARPS x
 // groups of four, 1M Gaussians 5 760 -> 3 815 us, 250K 1 445 -> 1 070 us, 100K
 // (400K entries a group) 654 -> 638 us, 30K 252 -> 472 us; four 1352x1014 views
 // one by one (bins of 2x2 tiles), 500K Gaussians 1 151 -> 819 us, 100K 303 ->
-// 500 us.
+// 500 us.  (The pairs are counted on the device; the host has the entries only.)
 constexpr int64_t CS_GROUP_ENTRIES = 400000;
 // Blocks of the counting sort's grid per SM, three of which are resident: the
 // resident blocks write into every list at once, each at its own depths, a few
@@ -1022,6 +1022,8 @@ __global__ void __launch_bounds__(CS_THREADS) cs_place_kernel(CsParams p)
 // catch up.  Whole binning, this way against the launches, in a graph / in a
 // stream: 1K entries 30 against 47 / 30 against 48 us, 16K 35 / 51 and 36 / 68,
 // 32K 43 / 53 and 44 / 71, 48K 51 / 53 and 56 / 73, 64K 59 / 53 and 63 / 75.
+// The line is the graph's, whose replays must not lose; in a stream 64K would
+// still gain.
 constexpr int DC_CTAS = 8, DC_THREADS = 1024, DC_WARPS = DC_THREADS / 32, DC_ROUNDS = 6;
 constexpr int DC_ROW = RADIX + 1;   // a digit's counters of 8 w rows meet different banks
 constexpr int64_t DC_MAX_ENTRIES = (int64_t)DC_CTAS * DC_THREADS * DC_ROUNDS;   // 49 152

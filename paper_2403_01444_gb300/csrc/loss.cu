@@ -25,14 +25,13 @@ namespace gs3 {
 // Of the squares only (x - y)^2 is filtered: sigma_x^2 + sigma_y^2 is its
 // variance plus twice the covariance, and written so the map's numerator and
 // denominator share the covariance's rounding.
-// Four planes of three channels, 1352x1014: 277 -> 198 us for the whole call
-// (pass 1 157 -> 99 us, pass 2 109 -> 91 us, pass 3 8 -> 5 us); one 479x361
-// image 26 -> 20 us, sixteen 1920x1080 images 1 500 -> 1 060 us; the
-// gradient's error against 64 bits 6.6e-6 -> 6.1e-6 relative.  The former form
-// filtered rows first with pairs along the row (extra additions, and twice
-// the weights, fetched again at each use), staged by TMA where W is a
-// multiple of 4.  Measured and not kept: both passes on chunks of planes whose
-// coefficients stay in L2 (222 us: the chunks' last waves cost more).
+// Four planes of three channels, 1352x1014: 191 us for the whole call (pass 1
+// 99, pass 2 90, pass 3 5 us); one 479x361 image 17 us, sixteen 1920x1080 images
+// 1 050 us; the gradient's error against 64 bits 6.1e-6 relative.  Rows first
+// with pairs along the row (extra additions, and twice the weights, fetched
+// again at each use), staged by TMA where W is a multiple of 4: 277, 26 and
+// 1 500 us, 6.6e-6.  Both passes on chunks of planes whose coefficients stay in
+// L2: 222 us (the chunks' last waves cost more).
 constexpr int LX = 54, LY = 32;      // outputs of a tile
 constexpr int LH = 5;                // window half-width
 constexpr int LC = LX + 2 * LH;      // columns of the column stage

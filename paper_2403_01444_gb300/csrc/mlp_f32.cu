@@ -194,10 +194,10 @@ __global__ void __launch_bounds__(MF_THREADS, 4) mlp_f32_fwd_kernel(const ET *en
 
 // One block runs the forward pass of a chunk again, then the row gradients
 // and the weight gradients.  These are summed in three levels, so that no chain
-// of additions grows with the rows of all chunks: a chunk's rows (the even and
-// the odd ones, 32 each; 8 a warp for the last layer), the chunks in registers
-// that live over all of them, and the blocks by one atomic a weight and block
-// at the end (the last layer's warps are added up before).
+// of additions runs over all rows of a block: a chunk's rows (the even and the
+// odd ones, 32 each; 8 a warp for the last layer), the chunks in registers that
+// live over all of them, and the blocks by one atomic a weight and block at the
+// end (the last layer's warps are added up before).
 template <typename ET>
 __global__ void __launch_bounds__(MF_THREADS, 2)
     mlp_f32_bwd_kernel(const ET *enc, bool vec, int64_t n, const float *W, const float *d_raw7, const float *d_scale,

@@ -129,14 +129,14 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_al
 // therefore run as a pipeline with one barrier each: while a batch of staged
 // records is composited, the next batch's candidates are in flight to
 // registers (their indices one batch earlier) and the colours of the records
-// just kept to shared memory (cp.async).  Before, each batch waited for its
-// indices, records and colours in turn, behind three barriers: 575 -> 523 us
-// at 250K Gaussians and four 1352x1014 views, 235 -> 189 us at 50K and eight
-// 480x360 views, 94 -> 67 us at 49K and one 477x363 view.  Measured slower:
-// four pixels a lane as in the reverse (676 / 272 / 95 us: it needs 120
-// registers, and fewer warps hide less), records culled per warp (576 / 204 /
-// 65 us), two candidates a thread per batch (745 / 255 / 78 us at 64
-// registers), no per-lane skip of records (548 / 223 / 78 us).
+// just kept to shared memory (cp.async).  250K Gaussians and four 1352x1014
+// views / 50K and eight 480x360 / 49K and one 477x363 view: 523 / 189 / 67 us.
+// Measured slower: a batch that waits for its indices, records and colours in
+// turn, behind three barriers (575 / 235 / 94 us), four pixels a lane as in the
+// reverse (676 / 272 / 95 us: it needs 120 registers, and fewer warps hide
+// less), records culled per warp (576 / 204 / 65 us), two candidates a thread
+// per batch (745 / 255 / 78 us at 64 registers), no per-lane skip of records
+// (548 / 223 / 78 us).
 constexpr int FWD_UNROLL = 4;
 
 struct FwdBatch {
@@ -351,20 +351,19 @@ __device__ __forceinline__ float rcp_approx(float x)
 
 // Reverse: one warp per 8x16 half of a tile, four vertically adjacent pixels a
 // lane as NP = 2 packed pairs (or 8x8 and NP = 1, see kFewTiles), no barrier
-// anywhere; the warps of a block share nothing.  What bounds it is the instruction issue of the pair arithmetic
-// and, at small images, the longest tile.  Why it is cut this way (250K
-// Gaussians, four 1352x1014 views / 50K, eight 480x360 views, one launch, by
-// CUPTI):
+// anywhere; the warps of a block share nothing.  What bounds it is the pair
+// arithmetic (FMA pipe 55 %, 62 % of the issue slots) and, at small images, the
+// longest tile.  Why it is cut this way (250K Gaussians, four 1352x1014 views /
+// 50K, eight 480x360 views, one launch, by CUPTI: 646 / 184 us):
 //  - the sums over pixels are taken with the lanes turned.  While a chunk of
 //    BWD_CHUNK records is walked, lane = pixel column, and each lane leaves
 //    the sums over its own four pixels (of dL/dpower times 1, dy, dy^2 and of
 //    the colour gradient) in shared memory; then lane = (record, pixels), and
 //    four lanes add up a record's 32 columns.  A shuffle butterfly per record
 //    for each pixel pair, summed over a tile's warps behind two barriers a
-//    chunk, took half of the kernel's instructions: 922 / 293 us, against
-//    646 / 184 us now.
+//    chunk, takes half of a kernel's instructions (922 / 293 us).
 //  - each warp keeps, of the tile's list, the records that can reach its own
-//    half (staged_hits), which the former per-tile staging could not use.
+//    half (staged_hits).
 //  - four pixels a lane share a record's loads and column offset: two pixels
 //    a lane (8x8 per warp) run into the shared-memory pipe (79 % of its
 //    wavefronts) where there are many tiles, 725 us against 640.
@@ -400,7 +399,10 @@ struct PixBwd {
 // 128x96 views (192 tiles) 129 -> 76 us; 50K, eight 480x360 views (5 520) 207
 // -> 184 us; 250K, one 1352x1014 view (5 440) 154 -> 158 us; 1M, one 1920x1080
 // view (8 160) 262 -> 295 us; 250K, two 1352x1014 views (10 880) 352 -> 390 us;
-// 50K, sixteen 480x360 views (11 040) 368 -> 348 us.
+// 50K, sixteen 480x360 views (11 040) 368 -> 348 us.  What decides is how long
+// the longest lists are against the work of all, which the host does not know:
+// by tiles alone one 1352x1014 view is on the wrong side by 4 us and sixteen
+// 480x360 views by 20.
 constexpr int kFewTiles = 40;
 
 struct BwdWarp {

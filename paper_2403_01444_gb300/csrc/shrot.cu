@@ -109,10 +109,12 @@ __device__ __forceinline__ void quat_rot(const float *q, float *R)
 // One thread per Gaussian, a warp's 32 coefficient rows (contiguous in global
 // memory) passed through shared memory in both directions so that every
 // global access is a whole line; an odd row stride keeps a lane's walk down
-// its own row free of bank conflicts.  Bound by HBM: at 250K Gaussians of
-// degree 3 it reads and writes 96 MB.  With a thread loading and storing its
-// row straight from global memory each access touched 32 lines: 74 us, now
-// 25 us (degree 2, 49K Gaussians: 9.6 us, now 3.7 us).
+// its own row free of bank conflicts.  At 250K Gaussians of degree 3 it reads
+// and writes 96 MB, 14 us at the memory's rate, and takes 25 us: 128 registers
+// and 25 KB of shared memory a block leave 14 warps an SM (issue 59 % of the
+// slots), too few to keep that many bytes in flight.  With a thread loading and
+// storing its row straight from global memory each access touches 32 lines:
+// 74 us (degree 2, 49K Gaussians: 9.6 us, here 3.7 us).
 template <int DEG>
 __global__ void __launch_bounds__(128) sh_rotate_kernel(const float4 *q_from, const float4 *q_to, const float *sh_in,
                                                         int64_t n, float *sh_out, ShRotParams P)
